@@ -21,7 +21,8 @@
 // knot computes.  Systems may move derivative work off the backward
 // recursion: the planar arm stores every knot's derivative block, the rigid
 // trees every knot's substep primals, computed before the pass one knot per
-// lane (per-knot scratch, a.dscr).  G = 1 (single-lane groups) keeps the
+// lane (per-knot scratch, a.dscr); the point mass and the Dubins car keep
+// theirs in the knots' gain records.  G = 1 (single-lane groups) keeps the
 // whole backward knot in registers (backward_lane).
 //
 // Arithmetic: R = double (FP64 mode) or float (mixed mode).  In mixed mode
@@ -241,9 +242,11 @@ struct Solver {
   static constexpr int NF = n + m + m * (n + 1) + kLo;    // forward record: x, u, K, k, x_lo
   static constexpr int PF = (NF + G - 1) / G;             // prefetch registers per lane (forward)
   // prefetch registers per lane (backward): the knot record x_k, u_k, or,
-  // for systems that store a derivative block per knot, that block
+  // for systems that store a derivative block per knot (in its own scratch or
+  // in the knot's gain record), that block
   template <class S> static constexpr int bwd_prefetch_elems() {
     if constexpr (S::kStoredDerivs) return S::kDerivStride;
+    else if constexpr (S::kGainDerivs) return S::kBlock;
     else return S::n + S::m;
   }
   static constexpr int PB = (bwd_prefetch_elems<Sys>() + G - 1) / G;
@@ -258,6 +261,12 @@ struct Solver {
   }
   static_assert(step_slots_fit<Sys>(), "line-search lanes exceed the system's step slots");
   static_assert(!Sys::kKnotParallel || G >= 32, "knot-parallel derivatives need groups of whole warps");
+  // where this lane's share of a gain-record block goes (the second: a
+  // symmetric pair's mirrored entry), the same at every knot
+  struct BlockDst {
+    R* d0[PB];
+    R* d1[PB];
+  };
   typedef typename Sys::template ParamsT<R> Params;
   static constexpr bool kLane = (G == 1);                  // one thread per instance, matrices in registers
   // lanes of a warp that are not a group's first lane (sub-warp groups)
@@ -835,9 +844,9 @@ struct Solver {
   // ------------------------------------------------------------------------
   TO_DEV static int backward_knot(const Params& P, const Group<G>& g, W& w, bool act, bool act_next,
                                   const SolveArgs& a, R (&pb)[PB], const R* trec_next, R* grec, double* vxrec,
-                                  double mu_lm, bool timer, long long& tlast, const R* kprim) {
+                                  double mu_lm, bool timer, long long& tlast, const R* kprim, const BlockDst& dst) {
     const R eps = (R)a.eps;
-    if constexpr (!Sys::kStoredDerivs) {   // x_k, u_k feed the derivative step (stored blocks need neither)
+    if constexpr (!Sys::kStoredDerivs && !Sys::kGainDerivs) {   // x_k, u_k feed the derivative step (stored blocks need neither)
       if (act) {
 #pragma unroll
         for (int s = 0; s < PB; ++s) {
@@ -883,11 +892,20 @@ struct Solver {
           if (e < DS) pb[s] = kprim[e];
         }
       }
+    } else if constexpr (Sys::kGainDerivs) {
+      // the knot's block from its gain record, prefetched into pb D knots
+      // earlier, to its places among the constants (block_consts, once a pass)
+#pragma unroll
+      for (int s = 0; s < PB; ++s) {
+        const int e = g.lane + s * G;
+        if (act && e < Sys::kBlock) {
+          *dst.d0[s] = pb[s];
+          *dst.d1[s] = pb[s];
+        }
+        if (act_next && e < Sys::kBlock) pb[s] = kprim[e];
+      }
     } else if (act) {
-      if constexpr (Sys::kKnotParallel)
-        Sys::template derivs_staged<R, G>(P, g, w.xk, w.uk, eps, w.A, w.Bm, w.lxx, w.lx, w.luu, w.lu, w.sx, kprim);
-      else
-        Sys::template derivs<R, G>(P, g, w.xk, w.uk, eps, w.A, w.Bm, w.lxx, w.lx, w.luu, w.lu, w.sx);
+      Sys::template derivs_staged<R, G>(P, g, w.xk, w.uk, eps, w.A, w.Bm, w.lxx, w.lx, w.luu, w.lu, w.sx, kprim);
     }
     g.sync();
     TO_TICK(1);
@@ -1396,7 +1414,7 @@ struct Solver {
               if (a.vx && a.want_vx)
                 for (int i = 0; i < n; ++i) vx_at(a, a.vx, base + T)[i] = (double)w.v[i];
             }
-            if constexpr (!Sys::kStoredDerivs) {
+            if constexpr (!Sys::kStoredDerivs && !Sys::kGainDerivs) {
 #pragma unroll
               for (int i = 0; i < D; ++i) {
                 if (T - 1 - i < 0) break;
@@ -1411,9 +1429,27 @@ struct Solver {
               }
             }
           }
-          if constexpr (Sys::kStoredDerivs) {
-            // every lane: the whole derivative block of its knots, stored
-            // (no barrier inside: the groups of a warp may run different T)
+          BlockDst dst;
+          if constexpr (Sys::kGainDerivs) {
+#pragma unroll
+            for (int s = 0; s < PB; ++s) {
+              dst.d0[s] = Sys::block_dst(g.lane + s * G, false, w.A, w.lxx, w.lx, w.lu);
+              dst.d1[s] = Sys::block_dst(g.lane + s * G, true, w.A, w.lxx, w.lx, w.lu);
+            }
+            if (bw) Sys::block_consts(P, g.lane, G, (R)a.eps, w.A, w.Bm, w.lxx, w.lx, w.luu);
+          }
+          if constexpr (Sys::kStoredDerivs || Sys::kGainDerivs) {
+            // every lane: the derivative block of its knots, stored
+            // (no barrier inside: the groups of a warp may run different T).
+            // The recursion is bound by its longest dependent chain, and the
+            // blocks depend on nothing in it: computed on one lane inside it
+            // (3 bumps' exp one after another, the clip's divide and roots),
+            // the point mass's and the car's took 41 % (float64) and 53 %
+            // (float32) of the solve.  Out of it: point mass B=1 float64
+            // 1.65 -> 1.14 ms (2 iterations), car B=2048 float64 9.75 -> 6.68
+            // ms (3 iterations, V_x), car B=8192 float32 0.95 -> 0.81 ms; the
+            // same bits.  The gain record is free until the pass writes it,
+            // so the workspace does not grow.
             if (bw) {
               const R eps = (R)a.eps;
               // the next knot's record is loaded (16-byte vectors) while this one computes
@@ -1426,10 +1462,17 @@ struct Solver {
 #pragma unroll
                 for (int i = 0; i < m; ++i) u[i] = nr[n + i];
                 if (k + G < T) ld_vec<RS>(rec(a, traj, base, k + G, cur), nr);
+                if constexpr (Sys::kGainDerivs) {
+                  static_assert(Sys::kBlockPad <= GS, "the block fits the gain record");
+                  R d[Sys::kBlockPad];
+                  Sys::block(P, x, u, eps, d);
+                  st_vec<Sys::kBlockPad>(grec_at(a, gains, base + k), d);
+                } else {
                 R d[Sys::kDerivStride];
                 Sys::derivs_lane(P, x, u, eps, d, d + n * n, d + n * n + n * m, d + 2 * n * n + n * m,
                                  d + 2 * n * n + n * m + n, d + 2 * n * n + n * m + n + m * m);
                 st_vec<Sys::kDerivStride>(dscr_at(a, base + k), d);
+                }
               }
             }
           }
@@ -1447,18 +1490,18 @@ struct Solver {
               }
           }
           g.sync();
-          if constexpr (Sys::kStoredDerivs) {
+          if constexpr (Sys::kStoredDerivs || Sys::kGainDerivs) {
             // the last D knots' stored blocks (written above by the group's lanes)
             if (bw)
 #pragma unroll
               for (int i = 0; i < D; ++i) {
                 if (T - 1 - i < 0) break;
-                const R* d = dscr_at(a, base + T - 1 - i);
+                const R* d = Sys::kGainDerivs ? grec_at(a, gains, base + T - 1 - i) : dscr_at(a, base + T - 1 - i);
                 ring(T - 1 - i, [&](R (&b)[PB]) {
 #pragma unroll
                   for (int s = 0; s < PB; ++s) {
                     const int e = g.lane + s * G;
-                    if (e < Sys::kDerivStride) b[s] = d[e];
+                    if (e < bwd_prefetch_elems<Sys>()) b[s] = d[e];
                   }
                 });
               }
@@ -1473,13 +1516,13 @@ struct Solver {
               const bool act_next = bw && k >= D && k - D < T;   // the knot whose record this slot takes next
               const long long kk = base + (act ? k : 0);
               const R* rn = rec(a, traj, base, act_next ? k - D : 0, cur);
-              // rigid trees: the knot's stored substep primals; planar arm: the
+              // rigid trees: the knot's stored substep primals; the others: the
               // stored derivative block of the knot D earlier (this knot's is in pb)
-              const long long kd = Sys::kStoredDerivs ? base + (act_next ? k - D : 0) : kk;
-              const R* kprim = (Sys::kKnotParallel || Sys::kStoredDerivs) ? dscr_at(a, kd) : nullptr;
+              const long long kd = Sys::kKnotParallel ? kk : base + (act_next ? k - D : 0);
+              const R* kprim = Sys::kGainDerivs ? grec_at(a, gains, kd) : dscr_at(a, kd);
               const int f = backward_knot(P, g, w, act, act_next, a, pb[d], rn, grec_at(a, gains, kk),
                                           (a.vx && a.want_vx && act) ? vx_at(a, a.vx, kk) : nullptr, mu_lm, timer,
-                                          tlast, kprim);
+                                          tlast, kprim, dst);
               if (f == 1) flags |= ST_FLAG_REG;
               // Levenberg-Marquardt: any failed factor (pivot test, or a
               // non-finite Q_uu once an earlier knot's gains were skipped)

@@ -71,12 +71,18 @@ struct SysDubins {
     return P.wpT * (x[0] * x[0] + x[1] * x[1]) + P.wvT * x[3] * x[3] + P.waT * x[4] * x[4];
   }
 
-  // Running-cost derivatives: the bumps act on the position block only, so
-  // the clipped 5x5 state Hessian is the clipped 2x2 position block with the
-  // clip of 0 on the other diagonal entries.  One lane.
+  // What a knot's derivatives hold besides constants, computed for every knot
+  // before the backward pass, one knot per lane, and kept in the knot's gain
+  // record (free until that knot's gains are written):
+  //   [0..3] A(0, 2), A(0, 3), A(1, 2), A(1, 3)  [4..6] the clipped position
+  //   block of l_xx (xx, xy, yy)  [7..8] l_x  [9..10] l_u  [11] padding
+  // The bumps act on the position block only, so the clipped 5x5 state Hessian
+  // is the clipped 2x2 position block with the clip of 0 on the other diagonal
+  // entries.
+  static constexpr bool kGainDerivs = true;
+  static constexpr int kBlock = 11, kBlockPad = 12;
   template <class R>
-  TO_DEV static void running_derivs(const ParamsT<R>& P, const R* x, const R* u, R eps, R* lxx, R* lx, R* luu,
-                                    R* lu) {
+  TO_DEV static void block(const ParamsT<R>& P, const R* x, const R* u, R eps, R* d) {
     R gx = 0, gy = 0, hxx = 0, hxy = 0, hyy = 0;
     const R is2 = R(1) / (P.bsig * P.bsig);
     const R inv = R(0.5) * is2;
@@ -90,62 +96,68 @@ struct SysDubins {
       hxy += es * dx * dy * is2;
     }
     eigclip_2x2(hxx, hxy, hyy, eps);
-#pragma unroll
-    for (int i = 0; i < n * n; ++i) lxx[i] = 0;
-    lxx[0] = hxx; lxx[1] = hxy; lxx[n] = hxy; lxx[n + 1] = hyy;
-    lxx[2 * n + 2] = clip0(eps); lxx[3 * n + 3] = clip0(eps); lxx[4 * n + 4] = clip0(eps);
-    lx[0] = gx; lx[1] = gy; lx[2] = 0; lx[3] = 0; lx[4] = 0;
-    const R w2 = R(2) * P.wu;
-    const R d = w2 > eps ? w2 : eps;
-    luu[0] = d; luu[1] = 0; luu[2] = 0; luu[3] = d;
-    lu[0] = w2 * u[0]; lu[1] = w2 * u[1];
-  }
-
-  // A = df/dx, B = df/du in closed form, entries spread over the lanes; the
-  // cost derivatives on the last lane of the group
-  template <class R, int G>
-  TO_DEV static void derivs(const ParamsT<R>& P, const Group<G>& g, const R* x, const R* u, R eps, R* A, R* B,
-                            R* lxx, R* lx, R* luu, R* lu, R*) {
     R s, c;
     sincos(x[2], &s, &c);
-    for (int e = g.lane; e < n * n + n * m; e += G) {
-      if (e < n * n) {
-        const int i = e / n, j = e % n;
-        R v = (i == j) ? R(1) : R(0);
-        if (i == 0 && j == 2) v = -P.dt * x[3] * s;
-        if (i == 0 && j == 3) v = P.dt * c;
-        if (i == 1 && j == 2) v = P.dt * x[3] * c;
-        if (i == 1 && j == 3) v = P.dt * s;
-        if (i == 3 && j == 4) v = P.dt;
-        A[e] = v;
-      } else {
-        const int f = e - n * n, i = f / m, j = f % m;
-        B[f] = ((i == 2 && j == 0) || (i == 4 && j == 1)) ? P.dt : R(0);
-      }
+    const R w2 = R(2) * P.wu;
+    d[0] = -P.dt * x[3] * s;
+    d[1] = P.dt * c;
+    d[2] = P.dt * x[3] * c;
+    d[3] = P.dt * s;
+    d[4] = hxx; d[5] = hxy; d[6] = hyy;
+    d[7] = gx; d[8] = gy;
+    d[9] = w2 * u[0]; d[10] = w2 * u[1];
+    d[11] = R(0);
+  }
+  // the constant entries: A, B, and l_xx, l_x, l_uu outside the block (lane
+  // of a group of G)
+  template <class R>
+  TO_DEV static void block_consts(const ParamsT<R>& P, int lane, int G, R eps, R* A, R* B, R* lxx, R* lx, R* luu) {
+    const R w2 = R(2) * P.wu;
+    for (int e = lane; e < n * n; e += G) {
+      const int i = e / n, j = e % n;
+      A[e] = (i == j) ? R(1) : ((i == 3 && j == 4) ? P.dt : R(0));
+      lxx[e] = (i == j && i >= 2) ? clip0(eps) : R(0);
     }
-    if (g.lane == G - 1) running_derivs(P, x, u, eps, lxx, lx, luu, lu);
+    for (int e = lane; e < n * m; e += G) B[e] = (e == 2 * m || e == 4 * m + 1) ? P.dt : R(0);
+    for (int e = lane; e < n; e += G) lx[e] = R(0);
+    for (int e = lane; e < m * m; e += G) luu[e] = (e / m == e % m) ? (w2 > eps ? w2 : eps) : R(0);
+  }
+  // where entry e of the block goes; the mirrored entry of a symmetric pair
+  // (second), else the same place
+  template <class R>
+  TO_DEV static R* block_dst(int e, bool second, R* A, R* lxx, R* lx, R* lu) {
+    return e < 4 ? A + (e >> 1) * n + 2 + (e & 1)
+                 : e == 4 ? lxx : e == 5 ? lxx + (second ? n : 1) : e == 6 ? lxx + n + 1 : e < 9 ? lx + (e - 7) : lu + (e - 9);
   }
 
-  // the same on one lane (single-lane groups)
+  // the whole derivatives on one lane (single-lane groups)
   template <class R>
   TO_DEV static void derivs_lane(const ParamsT<R>& P, const R* x, const R* u, R eps, R* A, R* B, R* lxx, R* lx,
                                  R* luu, R* lu) {
-    R s, c;
-    sincos(x[2], &s, &c);
+    R d[kBlockPad];
+    block(P, x, u, eps, d);
 #pragma unroll
     for (int i = 0; i < n; ++i)
 #pragma unroll
       for (int j = 0; j < n; ++j) A[i * n + j] = (i == j) ? R(1) : R(0);
-    A[0 * n + 2] = -P.dt * x[3] * s;
-    A[0 * n + 3] = P.dt * c;
-    A[1 * n + 2] = P.dt * x[3] * c;
-    A[1 * n + 3] = P.dt * s;
+    A[0 * n + 2] = d[0];
+    A[0 * n + 3] = d[1];
+    A[1 * n + 2] = d[2];
+    A[1 * n + 3] = d[3];
     A[3 * n + 4] = P.dt;
 #pragma unroll
     for (int i = 0; i < n * m; ++i) B[i] = R(0);
     B[2 * m + 0] = P.dt;
     B[4 * m + 1] = P.dt;
-    running_derivs(P, x, u, eps, lxx, lx, luu, lu);
+#pragma unroll
+    for (int i = 0; i < n * n; ++i) lxx[i] = 0;
+    lxx[0] = d[4]; lxx[1] = d[5]; lxx[n] = d[5]; lxx[n + 1] = d[6];
+    lxx[2 * n + 2] = clip0(eps); lxx[3 * n + 3] = clip0(eps); lxx[4 * n + 4] = clip0(eps);
+    lx[0] = d[7]; lx[1] = d[8]; lx[2] = 0; lx[3] = 0; lx[4] = 0;
+    const R w2 = R(2) * P.wu;
+    const R q = w2 > eps ? w2 : eps;
+    luu[0] = q; luu[1] = 0; luu[2] = 0; luu[3] = q;
+    lu[0] = d[9]; lu[1] = d[10];
   }
 
   template <class R>

@@ -52,6 +52,7 @@ struct SysPlanar3 {
   // derivatives computed for every knot before the backward pass, one knot
   // per lane (derivs_lane), and stored: A, B, l_xx, l_x, l_uu, l_u
   static constexpr bool kStoredDerivs = true;
+  static constexpr bool kGainDerivs = false;
   static constexpr int kDerivStride = n * n + n * m + n * n + n + m * m + m;
 
   // absolute link angles, link and centre-of-mass vectors, joint positions

@@ -63,13 +63,18 @@ struct SysPointMass {
     return P.wpT * (x[0] * x[0] + x[1] * x[1]) + P.wvT * (x[2] * x[2] + x[3] * x[3]);
   }
 
-  // Running-cost derivatives with the state and control Hessians clipped.
+  // What a knot's derivatives hold besides constants, computed for every knot
+  // before the backward pass, one knot per lane, and kept in the knot's gain
+  // record (free until that knot's gains are written):
+  //   [0..2] the clipped position block of l_xx (xx, xy, yy)  [3..4] l_x
+  //   [5..6] l_u  [7] padding
   // The bumps act on the position block only, so the clip of the full 4x4
   // state Hessian is the clip of the 2x2 position block with eps on the
-  // velocity diagonal (the remaining eigenpairs are (0, e_i)).  One lane.
+  // velocity diagonal (the remaining eigenpairs are (0, e_i)).
+  static constexpr bool kGainDerivs = true;
+  static constexpr int kBlock = 7, kBlockPad = 8;
   template <class R>
-  TO_DEV static void running_derivs(const ParamsT<R>& P, const R* x, const R* u, R eps, R* lxx, R* lx, R* luu,
-                                    R* lu) {
+  TO_DEV static void block(const ParamsT<R>& P, const R* x, const R* u, R eps, R* d) {
     R gx = 0, gy = 0, hxx = 0, hxy = 0, hyy = 0;
     const R s2 = P.bsig * P.bsig;
     const R is2 = R(1) / s2;
@@ -86,38 +91,39 @@ struct SysPointMass {
       hxy += es * dx * dy * is2;
     }
     eigclip_2x2(hxx, hxy, hyy, eps);
-#pragma unroll
-    for (int i = 0; i < n * n; ++i) lxx[i] = 0;
-    lxx[0] = hxx; lxx[1] = hxy; lxx[4] = hxy; lxx[5] = hyy;
-    lxx[10] = clip0(eps); lxx[15] = clip0(eps);
-    lx[0] = gx; lx[1] = gy; lx[2] = 0; lx[3] = 0;
     const R w2 = R(2) * P.wu;
-    const R d = w2 > eps ? w2 : eps;
-    luu[0] = d; luu[1] = 0; luu[2] = 0; luu[3] = d;
-    lu[0] = w2 * u[0]; lu[1] = w2 * u[1];
+    d[0] = hxx; d[1] = hxy; d[2] = hyy;
+    d[3] = gx; d[4] = gy;
+    d[5] = w2 * u[0]; d[6] = w2 * u[1];
+    d[7] = R(0);
   }
-
-  // A, B (row-major, constant) on every lane; the cost derivatives on the
-  // last lane of the group
-  template <class R, int G>
-  TO_DEV static void derivs(const ParamsT<R>& P, const Group<G>& g, const R* x, const R* u, R eps, R* A, R* B,
-                            R* lxx, R* lx, R* luu, R* lu, R*) {
-    for (int e = g.lane; e < n * n + n * m; e += G) {
-      if (e < n * n) {
-        int i = e / n, j = e % n;
-        A[e] = (i == j) ? R(1) : ((j == i + 2) ? P.dt : R(0));
-      } else {
-        int f = e - n * n, i = f / m, j = f % m;
-        B[f] = (i == j + 2) ? P.dt : R(0);
-      }
+  // the constant entries: A, B, and l_xx, l_x, l_uu outside the block (lane
+  // of a group of G)
+  template <class R>
+  TO_DEV static void block_consts(const ParamsT<R>& P, int lane, int G, R eps, R* A, R* B, R* lxx, R* lx, R* luu) {
+    const R w2 = R(2) * P.wu;
+    for (int e = lane; e < n * n; e += G) {
+      const int i = e / n, j = e % n;
+      A[e] = (i == j) ? R(1) : ((j == i + 2) ? P.dt : R(0));
+      lxx[e] = (i == j && i >= 2) ? clip0(eps) : R(0);
     }
-    if (g.lane == G - 1) running_derivs(P, x, u, eps, lxx, lx, luu, lu);
+    for (int e = lane; e < n * m; e += G) B[e] = (e / m == e % m + 2) ? P.dt : R(0);
+    for (int e = lane; e < n; e += G) lx[e] = R(0);
+    for (int e = lane; e < m * m; e += G) luu[e] = (e / m == e % m) ? (w2 > eps ? w2 : eps) : R(0);
+  }
+  // where entry e of the block goes; the mirrored entry of a symmetric pair
+  // (second), else the same place
+  template <class R>
+  TO_DEV static R* block_dst(int e, bool second, R*, R* lxx, R* lx, R* lu) {
+    return e == 0 ? lxx : e == 1 ? lxx + (second ? n : 1) : e == 2 ? lxx + n + 1 : e < 5 ? lx + (e - 3) : lu + (e - 5);
   }
 
-  // the same on one lane (single-lane groups)
+  // the whole derivatives on one lane (single-lane groups)
   template <class R>
   TO_DEV static void derivs_lane(const ParamsT<R>& P, const R* x, const R* u, R eps, R* A, R* B, R* lxx, R* lx,
                                  R* luu, R* lu) {
+    R d[kBlockPad];
+    block(P, x, u, eps, d);
 #pragma unroll
     for (int i = 0; i < n; ++i)
 #pragma unroll
@@ -126,7 +132,15 @@ struct SysPointMass {
     for (int i = 0; i < n; ++i)
 #pragma unroll
       for (int j = 0; j < m; ++j) B[i * m + j] = (i == j + 2) ? P.dt : R(0);
-    running_derivs(P, x, u, eps, lxx, lx, luu, lu);
+#pragma unroll
+    for (int i = 0; i < n * n; ++i) lxx[i] = 0;
+    lxx[0] = d[0]; lxx[1] = d[1]; lxx[n] = d[1]; lxx[n + 1] = d[2];
+    lxx[2 * n + 2] = clip0(eps); lxx[3 * n + 3] = clip0(eps);
+    lx[0] = d[3]; lx[1] = d[4]; lx[2] = 0; lx[3] = 0;
+    const R w2 = R(2) * P.wu;
+    const R q = w2 > eps ? w2 : eps;
+    luu[0] = q; luu[1] = 0; luu[2] = 0; luu[3] = q;
+    lu[0] = d[5]; lu[1] = d[6];
   }
 
   template <class R>

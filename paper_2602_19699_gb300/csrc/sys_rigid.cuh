@@ -772,6 +772,7 @@ struct SysRigid {
   // pass at once (derivs_staged).  No lane waits for a primal.
   static constexpr bool kKnotParallel = true;
   static constexpr bool kStoredDerivs = false;
+  static constexpr bool kGainDerivs = false;
   // elements per stored substep primal (a whole number of 16-byte chunks)
   template <class R> static constexpr int kPrimStride = (int)(((sizeof(Prim<R>) + 15) / 16 * 16) / sizeof(R));
 
