@@ -176,7 +176,9 @@ typedef struct {
                              sizes (1/8/16/32 point mass and Dubins car,
                              1/4/8/16/32 planar arm, 32 arm, 64/32
                              quadruped); 0 = the totune
-                             choice, else the system's default.  1: one thread
+                             choice, else the system's default for the batch
+                             size (planar arm: 16 for float32 batches that
+                             would leave SMs idle at 8).  1: one thread
                              per instance with every per-knot matrix in
                              registers; its line search tries one step size
                              at a time (the smallest j first), the others

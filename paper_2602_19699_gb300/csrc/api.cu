@@ -446,6 +446,13 @@ static int resolve_shape(to_problem p, const to_solver_opts* o, int B, double fr
     depth = p->tuned_depth[prec];
   }
   if (!depth) depth = 1;
+  int dev = 0, sms = 0;
+  TO_CK(cudaGetDevice(&dev));
+  TO_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (!G && !gpb && ops->lanes) {
+    G = ops->lanes(prec, B, std::max(1, (int)(sms * std::min(1.0, std::max(frac, 0.0)))));
+    if (G != ops->default_G) gpb = std::max(1, 64 / G);
+  }
   if (!G) G = ops->default_G;
   if (!gpb) {
     gpb = ops->default_gpb[prec];
@@ -463,9 +470,6 @@ static int resolve_shape(to_problem p, const to_solver_opts* o, int B, double fr
   int bps = 0;
   TO_CK(ops->occupancy(prec, G, depth, gpb, &smem, &bps));
   if (bps < 1) return fail(TO_ERR_ARG, "opts: launch shape does not fit on an SM");
-  int dev = 0, sms = 0;
-  TO_CK(cudaGetDevice(&dev));
-  TO_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int cap = std::max(1, (int)(bps * sms * std::min(1.0, std::max(frac, 0.0))));
   *G_out = G;
   *gpb_out = gpb;

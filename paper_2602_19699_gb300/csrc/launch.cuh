@@ -27,6 +27,11 @@ struct SysOps {
   int n_groups;                     // supported group sizes
   int groups[6];
   int default_G, default_gpb[2];    // default launch shape (FP64, mixed)
+  // lanes per instance of a solve of B instances on sms SMs that names no
+  // shape; null: default_G.  The sizes it picks from give the same bits (a
+  // result does not depend on the batch it is solved in), and each other
+  // size's CTAs have 64 threads
+  int (*lanes)(int prec, int B, int sms);
   bool accepts_actor;
   // parse the flat parameter vector into the system's struct in float64 and float32
   int (*parse)(const double* p, size_t np, std::vector<unsigned char>& blob64, std::vector<unsigned char>& blob32,

@@ -61,6 +61,16 @@ static cudaError_t planar3_occupancy(int prec, int G, int depth, int gpb, size_t
 // every knot's stored derivative block (both precisions)
 static size_t planar3_knot_scratch(const double*, size_t, int) { return SysPlanar3::kDerivStride; }
 
+// Float32 batches that leave SMs idle at 8 lanes take 16: the 16 step sizes
+// then take one line-search round, and a warp's instances (2, not 4) wait for
+// each other's second round no more.  Measured (T 100..400, 3 iterations, ms
+// at 8 / 16 lanes): B = 64 4.46 / 3.30, 608 4.88 / 3.68, 2432 5.55 / 4.53,
+// 3000 6.19 / 4.56, 4000 6.70 / 6.02, 5000 6.77 / 7.14, 8192 8.76 / 11.2; 1.5
+// times the 16 instances an SM holds at once is where the batch still pays.
+// Both sizes give the same bits in float32.  In float64 they do not (the
+// compiler fuses other multiply-adds), and the arm amplifies it.
+static int planar3_lanes(int prec, int B, int sms) { return prec == PREC_MIXED && B <= 24 * sms ? 16 : 8; }
+
 static SysOps make_ops() {
   SysOps o{};
   o.sys = 2;
@@ -70,6 +80,7 @@ static SysOps make_ops() {
   o.groups[4] = 4;   // stored derivatives need no lane per derivative role
   o.default_G = 8;
   o.default_gpb[0] = 8; o.default_gpb[1] = 8;
+  o.lanes = planar3_lanes;
   o.accepts_actor = false;
   o.parse = parse_planar3;
   o.max_depth = 2;   // groups of 4 or more lanes

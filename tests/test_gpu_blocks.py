@@ -36,7 +36,7 @@ def test_gains_match_the_oracle(P, oracle_mod, make, prec, G):
     o = oracle_mod.Oracle.from_problem(prob)
     tol = 1e-11 if prec == "fp64" else 1e-3
     done = (r["status"] & 15) == P.TO_ST_MAX_ITER       # V_x and K belong to the returned iterate
-    assert done.mean() > 0.8
+    assert done[T >= 7].all()       # (the car cannot move its position in one or two knots from rest)
     for i in np.flatnonzero(done):
         t = int(T[i])
         K, _, Vx, rc = o.backward(r["X"][i, :t + 1], r["U"][i, :t])
