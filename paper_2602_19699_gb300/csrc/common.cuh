@@ -159,6 +159,36 @@ TO_DEV bool dgt_nonneg(double s, double t) {
   return a > b && a < 0x7ff0000000000000LL;
 }
 
+// The Gaussian bumps around (px, py): use(dx, dy, e) for every bump in order,
+// e = exp(-(dx^2 + dy^2) inv).  In float32 the exponentials of up to four bumps
+// are evaluated side by side before the first is used, so their latencies
+// overlap.  In float64 there is nothing to overlap: an instruction holds the
+// scheduler's FP64 pipe for as long as its result takes (64 cycles), so they
+// follow one another in less code.
+template <int C, class R, class U>
+TO_DEV void bump_chunk(const R (*bc)[2], R px, R py, R inv, U& use) {
+  R dx[C], dy[C], e[C];
+#pragma unroll
+  for (int i = 0; i < C; ++i) {
+    dx[i] = px - bc[i][0];
+    dy[i] = py - bc[i][1];
+    e[i] = exp(-(dx[i] * dx[i] + dy[i] * dy[i]) * inv);
+  }
+#pragma unroll
+  for (int i = 0; i < C; ++i) use(dx[i], dy[i], e[i]);
+}
+template <class R, class U>
+TO_DEV void each_bump(const R (*bc)[2], int nb, R px, R py, R inv, U&& use) {
+  if constexpr (sizeof(R) == 8) {
+    for (int b = 0; b < nb; ++b) bump_chunk<1>(bc + b, px, py, inv, use);
+    return;
+  }
+  for (; nb >= 4; nb -= 4, bc += 4) bump_chunk<4>(bc, px, py, inv, use);
+  if (nb == 3) bump_chunk<3>(bc, px, py, inv, use);
+  else if (nb == 2) bump_chunk<2>(bc, px, py, inv, use);
+  else if (nb == 1) bump_chunk<1>(bc, px, py, inv, use);
+}
+
 // Unit eigenvector of the symmetric 3x3 A for the eigenvalue lam: the largest
 // cross product of two rows of A - lam I (they span the orthogonal complement
 // when lam is simple).

@@ -18,6 +18,7 @@ static int parse_dubins(const double* p, size_t np, std::vector<unsigned char>& 
   P.wpT = p[5 + 2 * P.nb];
   P.wvT = p[6 + 2 * P.nb];
   P.waT = p[7 + 2 * P.nb];
+  P.derive();
   to_blobs<DubinsParams>(P, blob64, blob32);
   return 0;
 }

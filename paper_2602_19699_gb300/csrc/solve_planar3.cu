@@ -38,6 +38,7 @@ static int parse_planar3(const double* p, size_t np, std::vector<unsigned char>&
   P.wee = c[10]; P.wvT = c[11];
   if ((int)c[12] != 2 || c[14] != 0 || c[15] != 0) { err = "planar3 params: end effector must be on link 3's x axis"; return -1; }
   P.len[2] = c[13];
+  P.derive();
   to_blobs<Planar3Params>(P, blob64, blob32);
   return 0;
 }

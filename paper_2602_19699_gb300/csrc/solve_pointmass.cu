@@ -17,6 +17,7 @@ static int parse_pointmass(const double* p, size_t np, std::vector<unsigned char
   for (int b = 0; b < P.nb; ++b) { P.bc[b][0] = p[5 + 2 * b]; P.bc[b][1] = p[6 + 2 * b]; }
   P.wpT = p[5 + 2 * P.nb];
   P.wvT = p[6 + 2 * P.nb];
+  P.derive();
   to_blobs<PointMassParams>(P, blob64, blob32);
   return 0;
 }

@@ -14,6 +14,13 @@ struct DubinsParams {
   R dt, wu, bamp, bsig, wpT, wvT, waT;
   int nb;
   R bc[8][2];
+  R is2, inv, inv2;   // 1 / sigma^2, half of it, 1 / (2 sigma^2)
+  // the quotients a rollout step would divide out again, rounded as there
+  void derive() {
+    is2 = R(1) / (bsig * bsig);
+    inv = R(0.5) * is2;
+    inv2 = R(1) / (R(2) * bsig * bsig);
+  }
 };
 
 template <class D, class S>
@@ -22,6 +29,7 @@ inline void cast_params(const DubinsParams<S>& s, DubinsParams<D>& d) {
   d.wpT = (D)s.wpT; d.wvT = (D)s.wvT; d.waT = (D)s.waT;
   d.nb = s.nb;
   for (int b = 0; b < 8; ++b) { d.bc[b][0] = (D)s.bc[b][0]; d.bc[b][1] = (D)s.bc[b][1]; }
+  d.derive();
 }
 
 struct SysDubins {
@@ -37,11 +45,7 @@ struct SysDubins {
   template <class R>
   TO_DEV static R bumps(const ParamsT<R>& P, R px, R py) {
     R s = 0;
-    const R inv = R(1) / (R(2) * P.bsig * P.bsig);
-    for (int b = 0; b < P.nb; ++b) {
-      const R dx = px - P.bc[b][0], dy = py - P.bc[b][1];
-      s += P.bamp * exp(-(dx * dx + dy * dy) * inv);
-    }
+    each_bump(P.bc, P.nb, px, py, P.inv2, [&](R, R, R e) { s += P.bamp * e; });
     return s;
   }
 
@@ -84,17 +88,15 @@ struct SysDubins {
   template <class R>
   TO_DEV static void block(const ParamsT<R>& P, const R* x, const R* u, R eps, R* d) {
     R gx = 0, gy = 0, hxx = 0, hxy = 0, hyy = 0;
-    const R is2 = R(1) / (P.bsig * P.bsig);
-    const R inv = R(0.5) * is2;
-    for (int b = 0; b < P.nb; ++b) {
-      const R dx = x[0] - P.bc[b][0], dy = x[1] - P.bc[b][1];
-      const R es = P.bamp * exp(-(dx * dx + dy * dy) * inv) * is2;
+    const R is2 = P.is2;
+    each_bump(P.bc, P.nb, x[0], x[1], P.inv, [&](R dx, R dy, R e) {
+      const R es = P.bamp * e * is2;
       gx -= es * dx;
       gy -= es * dy;
       hxx += es * (dx * dx * is2 - R(1));
       hyy += es * (dy * dy * is2 - R(1));
       hxy += es * dx * dy * is2;
-    }
+    });
     eigclip_2x2(hxx, hxy, hyy, eps);
     R s, c;
     sincos(x[2], &s, &c);

@@ -28,6 +28,15 @@ struct Planar3Params {
   int nb;
   R bc[2][2];
   R tgt[2];
+  R is2, inv, inv1, inv2;   // 1 / sigma^2, half of it, 0.5 / sigma^2, 1 / (2 sigma^2)
+  // the quotients a rollout step would divide out again, rounded as there
+  void derive() {
+    const R s2 = bsig * bsig;
+    is2 = R(1) / s2;
+    inv = R(0.5) * is2;
+    inv1 = R(0.5) / s2;
+    inv2 = R(1) / (R(2) * bsig * bsig);
+  }
 };
 
 template <class D, class S>
@@ -40,6 +49,7 @@ inline void cast_params(const Planar3Params<S>& s, Planar3Params<D>& d) {
   d.nb = s.nb;
   for (int b = 0; b < 2; ++b) { d.bc[b][0] = (D)s.bc[b][0]; d.bc[b][1] = (D)s.bc[b][1]; }
   d.tgt[0] = (D)s.tgt[0]; d.tgt[1] = (D)s.tgt[1];
+  d.derive();
 }
 
 struct SysPlanar3 {
@@ -239,11 +249,7 @@ struct SysPlanar3 {
     Kin<R> k;
     kinematics(P, xh, k);
     R l = P.wtau * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    const R inv = R(0.5) / (P.bsig * P.bsig);
-    for (int b = 0; b < P.nb; ++b) {
-      R dx = k.P[3][0] - P.bc[b][0], dy = k.P[3][1] - P.bc[b][1];
-      l += P.bamp * exp(-(dx * dx + dy * dy) * inv);
-    }
+    each_bump(P.bc, P.nb, k.P[3][0], k.P[3][1], P.inv1, [&](R, R, R e) { l += P.bamp * e; });
     R qdd[3], L[9];
     forward_dynamics(P, k, xh + 3, u, qdd, L);
     semi_implicit2<R, 3>(xh, xl, xh + 3, xl + 3, qdd, P.dt);
@@ -297,11 +303,7 @@ struct SysPlanar3 {
     Kin<R> k;
     kinematics(P, x, k);
     R l = P.wtau * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    const R inv = R(1) / (R(2) * P.bsig * P.bsig);
-    for (int b = 0; b < P.nb; ++b) {
-      R dx = k.P[3][0] - P.bc[b][0], dy = k.P[3][1] - P.bc[b][1];
-      l += P.bamp * exp(-(dx * dx + dy * dy) * inv);
-    }
+    each_bump(P.bc, P.nb, k.P[3][0], k.P[3][1], P.inv2, [&](R, R, R e) { l += P.bamp * e; });
     return l;
   }
 
@@ -319,18 +321,16 @@ struct SysPlanar3 {
     R ee[2], J[2][3];
     ee_derivs(k, ee, J);
     R gee[2] = {0, 0}, H[2][2] = {{0, 0}, {0, 0}};
-    const R s2 = P.bsig * P.bsig;
-    const R is2 = R(1) / s2, inv = R(0.5) * is2;
-    for (int b = 0; b < P.nb; ++b) {
-      const R d0 = ee[0] - P.bc[b][0], d1 = ee[1] - P.bc[b][1];
-      const R e = P.bamp * exp(-(d0 * d0 + d1 * d1) * inv);
+    const R is2 = P.is2;
+    each_bump(P.bc, P.nb, ee[0], ee[1], P.inv, [&](R d0, R d1, R ex) {
+      const R e = P.bamp * ex;
       const R g0 = d0 * is2, g1 = d1 * is2;     // gradient of the exponent / -1
       gee[0] -= e * g0;
       gee[1] -= e * g1;
       H[0][0] += e * (g0 * g0 - is2);
       H[1][1] += e * (g1 * g1 - is2);
       H[0][1] += e * g0 * g1;
-    }
+    });
     H[1][0] = H[0][1];
     assemble_q_block(k, ee, J, gee, H, eps, lxx, lx);
 #pragma unroll

@@ -11,6 +11,13 @@ struct PointMassParams {
   R dt, wu, bamp, bsig, wpT, wvT;
   int nb;
   R bc[8][2];
+  R is2, inv, inv2;   // 1 / sigma^2, half of it, 1 / (2 sigma^2)
+  // the quotients a rollout step would divide out again, rounded as there
+  void derive() {
+    is2 = R(1) / (bsig * bsig);
+    inv = R(0.5) * is2;
+    inv2 = R(1) / (R(2) * bsig * bsig);
+  }
 };
 
 template <class D, class S>
@@ -18,6 +25,7 @@ inline void cast_params(const PointMassParams<S>& s, PointMassParams<D>& d) {
   d.dt = (D)s.dt; d.wu = (D)s.wu; d.bamp = (D)s.bamp; d.bsig = (D)s.bsig; d.wpT = (D)s.wpT; d.wvT = (D)s.wvT;
   d.nb = s.nb;
   for (int b = 0; b < 8; ++b) { d.bc[b][0] = (D)s.bc[b][0]; d.bc[b][1] = (D)s.bc[b][1]; }
+  d.derive();
 }
 
 struct SysPointMass {
@@ -33,11 +41,7 @@ struct SysPointMass {
   template <class R>
   TO_DEV static R bumps(const ParamsT<R>& P, R px, R py) {
     R s = 0;
-    const R inv = R(1) / (R(2) * P.bsig * P.bsig);
-    for (int b = 0; b < P.nb; ++b) {
-      R dx = px - P.bc[b][0], dy = py - P.bc[b][1];
-      s += P.bamp * exp(-(dx * dx + dy * dy) * inv);
-    }
+    each_bump(P.bc, P.nb, px, py, P.inv2, [&](R, R, R e) { s += P.bamp * e; });
     return s;
   }
 
@@ -76,12 +80,9 @@ struct SysPointMass {
   template <class R>
   TO_DEV static void block(const ParamsT<R>& P, const R* x, const R* u, R eps, R* d) {
     R gx = 0, gy = 0, hxx = 0, hxy = 0, hyy = 0;
-    const R s2 = P.bsig * P.bsig;
-    const R is2 = R(1) / s2;
-    const R inv = R(0.5) * is2;
-    for (int b = 0; b < P.nb; ++b) {
-      R dx = x[0] - P.bc[b][0], dy = x[1] - P.bc[b][1];
-      R e = P.bamp * exp(-(dx * dx + dy * dy) * inv);
+    const R is2 = P.is2;
+    each_bump(P.bc, P.nb, x[0], x[1], P.inv, [&](R dx, R dy, R ex) {
+      const R e = P.bamp * ex;
       // d/dp e = -e d / s2 ;  d2/dp2 e = e (d d^T / s2^2 - I / s2)
       const R es = e * is2;
       gx -= es * dx;
@@ -89,7 +90,7 @@ struct SysPointMass {
       hxx += es * (dx * dx * is2 - R(1));
       hyy += es * (dy * dy * is2 - R(1));
       hxy += es * dx * dy * is2;
-    }
+    });
     eigclip_2x2(hxx, hxy, hyy, eps);
     const R w2 = R(2) * P.wu;
     d[0] = hxx; d[1] = hxy; d[2] = hyy;
