@@ -170,10 +170,26 @@ def totune(problem: "Problem", x0, T, opts: "to_solver_opts", max_rows: int = 64
              "ctas_per_sm": r.ctas_per_sm, "ms": r.ms, "stage_depth": r.stage_depth} for r in rows[:n.value]]
 
 
+class _Staging:
+    """Owner of a captured graph and its pinned staging: the graph object and
+    every view of the staging hold it, so a view outlives the graph object."""
+
+    def __init__(self, handle, batches):
+        self.handle, self.batches = handle, batches
+
+    def close(self):
+        if self.handle.value and _lib is not None:
+            _lib.tograph_destroy(self.handle)
+            self.handle.value = None
+
+    def __del__(self):
+        self.close()
+
+
 class Graph:
     """A captured multi-system solve (one member batch per problem).  Fill
     ``inputs(i)`` (pinned x0, T views), ``launch()``, ``sync()``, read
-    ``outputs(i)`` (pinned views, valid until the next launch)."""
+    ``outputs(i)`` (pinned views, valid until the next launch or ``close()``)."""
 
     def __init__(self, batches, B, opts: "to_solver_opts | None" = None, shares=None, want_traj: bool = True):
         self.batches = list(batches)
@@ -185,6 +201,7 @@ class Graph:
         self.want_traj = bool(want_traj)
         _check(lib().tograph_create(hb, Bs, sh, len(self.batches), C.byref(opts) if opts else None,
                                     int(self.want_traj), C.byref(self.handle)))
+        self._staging = _Staging(self.handle, self.batches)
         self._views = [self._member_views(i) for i in range(len(self.batches))]
         for bt, Bi in zip(self.batches, self.B):
             bt.B = Bi
@@ -199,8 +216,9 @@ class Graph:
         def view(p, shape, ctype, dtype):
             if not p.value:
                 return None
-            n = int(np.prod(shape))
-            return np.ctypeslib.as_array(C.cast(p, C.POINTER(ctype)), shape=(n,)).view(dtype).reshape(shape)
+            buf = (ctype * int(np.prod(shape))).from_address(p.value)
+            buf.owner = self._staging
+            return np.frombuffer(buf, dtype=dtype).reshape(shape)
         return {"x0": view(ptrs[0], (B, prob.n), C.c_double, np.float64),
                 "T": view(ptrs[1], (B,), C.c_int, np.int32),
                 "X": view(ptrs[2], (B, prob.T_max + 1, prob.n), C.c_double, np.float64),
@@ -227,12 +245,8 @@ class Graph:
         return lib().tograph_launch_count(self.handle)
 
     def close(self):
-        if getattr(self, "handle", None) and self.handle.value and _lib is not None:
-            _lib.tograph_destroy(self.handle)
-            self.handle = C.c_void_p()
-
-    def __del__(self):
-        self.close()
+        if getattr(self, "_staging", None) is not None:
+            self._staging.close()
 
 
 class Server:
