@@ -96,6 +96,12 @@ TO_DEV void semi_implicit2(R* qh, R* ql, R* vh, R* vl, const R* a, R h) {
   }
 }
 
+// products and multiply-adds that the compiler must not fuse otherwise
+TO_DEV float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+TO_DEV double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+TO_DEV float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+TO_DEV double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // clip of a zero eigenvalue, max(0, eps): the value a Hessian's entries
 // outside a cost's support take (0 when clipping is off, eps < 0)
 template <class R> TO_DEV R clip0(R eps) { return eps > R(0) ? eps : R(0); }

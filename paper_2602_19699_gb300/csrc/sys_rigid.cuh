@@ -162,6 +162,43 @@ struct SysRigid {
     const S c0 = a[1] * b[2] - a[2] * b[1], c1 = a[2] * b[0] - a[0] * b[2], c2 = a[0] * b[1] - a[1] * b[0];
     c[0] = c0; c[1] = c1; c[2] = c2;
   }
+  // y += a x b and y -= a x b.  In float64 fused: 6 operations, each of which
+  // holds the scheduler's FP64 pipe for 64 cycles, where the compiler makes 9.
+  // In float32 as the compiler fuses them: the arms are chaotic there, and
+  // their bits are kept.
+  template <class S> TO_DEV static void cross_acc(const S* a, const S* b, S* y) {
+    if constexpr (sizeof(S) == 8) {
+      y[0] = fma_rn(a[1], b[2], fma_rn(-a[2], b[1], y[0]));
+      y[1] = fma_rn(a[2], b[0], fma_rn(-a[0], b[2], y[1]));
+      y[2] = fma_rn(a[0], b[1], fma_rn(-a[1], b[0], y[2]));
+    } else {
+      y[0] += a[1] * b[2] - a[2] * b[1];
+      y[1] += a[2] * b[0] - a[0] * b[2];
+      y[2] += a[0] * b[1] - a[1] * b[0];
+    }
+  }
+  template <class S> TO_DEV static void cross_sub(const S* a, const S* b, S* y) {
+    if constexpr (sizeof(S) == 8) {
+      cross_acc(b, a, y);
+    } else {
+      S c[3];
+      cross(a, b, c);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) y[k] -= c[k];
+    }
+  }
+  // y += a x (s e_ax): a joint's own motion is along one axis, so 4 of the 6
+  // products of cross_acc would multiply by zero (which the compiler may not
+  // drop: 0 x is not 0 for every x)
+  template <class S> TO_DEV static S axpy(S a, S b, S y) {
+    if constexpr (sizeof(S) == 8) return fma_rn(a, b, y);
+    else return y + mul_rn(a, b);
+  }
+  template <class S> TO_DEV static void axis_acc(const S* a, int ax, S s, S* y) {
+    if (ax == 0) { y[1] = axpy(a[2], s, y[1]); y[2] = axpy(-a[1], s, y[2]); }
+    else if (ax == 1) { y[0] = axpy(-a[2], s, y[0]); y[2] = axpy(a[0], s, y[2]); }
+    else { y[0] = axpy(a[1], s, y[0]); y[1] = axpy(-a[0], s, y[1]); }
+  }
   // y = E x and y = E^T x for a row-major 3x3 E
   template <class S> TO_DEV static void mv(const S* E, const S* x, S* y) {
     const S y0 = E[0] * x[0] + E[1] * x[1] + E[2] * x[2];
@@ -197,6 +234,26 @@ struct SysRigid {
       case 2: { const S c = E[0], s = E[1]; y[0] = c * x0 - s * x1; y[1] = c * x1 + s * x0; y[2] = x2; break; }
       default: y[0] = x0; y[1] = x1; y[2] = x2;
     }
+  }
+
+  // Entry (r, k) of E M, of M E and of E^T M for a joint transform E (M
+  // row-major 3x3): a rotation about a coordinate axis leaves one row or column
+  // alone and mixes the other two (the identity, prismatic, none), so a product
+  // takes 12 multiply-adds where the full 3x3 one takes 27.
+  template <class R> TO_DEV static R e_row(int jt, const R* E, const R* M, int r, int k) {
+    if (jt > 2 || r == jt) return M[r * 3 + k];
+    const int i = (jt + 1) % 3, j = (jt + 2) % 3;
+    return E[r * 3 + i] * M[i * 3 + k] + E[r * 3 + j] * M[j * 3 + k];
+  }
+  template <class R> TO_DEV static R e_col(int jt, const R* M, const R* E, int r, int k) {
+    if (jt > 2 || k == jt) return M[r * 3 + k];
+    const int i = (jt + 1) % 3, j = (jt + 2) % 3;
+    return M[r * 3 + i] * E[i * 3 + k] + M[r * 3 + j] * E[j * 3 + k];
+  }
+  template <class R> TO_DEV static R et_row(int jt, const R* E, const R* M, int r, int k) {
+    if (jt > 2 || r == jt) return M[r * 3 + k];
+    const int i = (jt + 1) % 3, j = (jt + 2) % 3;
+    return E[i * 3 + r] * M[i * 3 + k] + E[j * 3 + r] * M[j * 3 + k];
   }
 
   // Plucker transform of joint i: E maps parent coordinates to body
@@ -255,79 +312,88 @@ struct SysRigid {
   template <class R, class S>
   TO_DEV static void inertia_mul(const ParamsT<R>& P, int i, const S* w, const S* v, S* n, S* f) {
     S c[3] = {S(P.com[i][0]), S(P.com[i][1]), S(P.com[i][2])};
-    S wc[3];
-    cross(w, c, wc);
     S p[3];
+    if constexpr (sizeof(S) == 8) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) p[k] = P.mass[i] * (v[k] + wc[k]);
-    S cp[3];
-    cross(c, p, cp);
+      for (int k = 0; k < 3; ++k) p[k] = v[k];
+      cross_acc(w, c, p);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) { n[k] = P.inertia[i][k] * w[k] + cp[k]; f[k] = p[k]; }
+      for (int k = 0; k < 3; ++k) { p[k] *= P.mass[i]; n[k] = P.inertia[i][k] * w[k]; f[k] = p[k]; }
+      cross_acc(c, p, n);
+    } else {
+      S wc[3];
+      cross(w, c, wc);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) p[k] = P.mass[i] * (v[k] + wc[k]);
+      S cp[3];
+      cross(c, p, cp);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) { n[k] = P.inertia[i][k] * w[k] + cp[k]; f[k] = p[k]; }
+    }
   }
 
-  // inverse dynamics: tau = ID(q, qd, qdd) with optional gravity and contact
+  // With the axis products and the sparse joint products (e_row), 7-DoF arm
+  // B=304 float64 17.2 -> 15.3 ms (V_x, 2 iterations), B=2048 float32 29.5 ->
+  // 27.5 ms (the same bits), quadruped B=512 float32 10.7 -> 9.5 ms.
+  // One body's velocity and its acceleration at qdd = 0, from its parent's
+  // (pa < 0: the fixed base, whose acceleration is -g): v and a transformed,
+  // the joint's own motion S qd, the velocity product v x (S qd); then the body
+  // force I a + v x* (I v).  Ept (nullable): the parent's linear velocity in
+  // body axes; Epw the angular one.
+  template <class R>
+  TO_DEV static void body_bias(const ParamsT<R>& P, int i, const R* E, const R* r, R qd, const R* pw, const R* pv,
+                               const R* paw, const R* pav, R* Epw, R* Ept, R* vw, R* vv, R* aw, R* av, R* hn, R* hf,
+                               R* fn, R* ff) {
+    const int pa = parent(i), jt = jtype(i), ax = jt <= 2 ? jt : jt - 3;
+    R t[3];
+    if (pa < 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) { Epw[k] = R(0); Ept[k] = R(0); aw[k] = R(0); t[k] = -P.g[k]; }
+    } else {
+      // X m = (E w, E (v - r x w))
+#pragma unroll
+      for (int k = 0; k < 3; ++k) t[k] = pv[k];
+      cross_sub(r, pw, t);
+      jmv(jt, E, pw, Epw);
+      jmv(jt, E, t, Ept);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) t[k] = pav[k];
+      cross_sub(r, paw, t);
+      jmv(jt, E, paw, aw);
+    }
+    jmv(jt, E, t, av);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { vw[k] = Epw[k]; vv[k] = Ept[k]; }
+    if (jt <= 2) vw[ax] += qd; else vv[ax] += qd;
+    if (pa >= 0) {
+      if (jt <= 2) {
+        axis_acc(vw, ax, qd, aw);
+        axis_acc(vv, ax, qd, av);
+      } else {
+        axis_acc(vw, ax, qd, av);
+      }
+    }
+    inertia_mul(P, i, aw, av, fn, ff);
+    inertia_mul(P, i, vw, vv, hn, hf);
+    cross_acc(vw, hn, fn);
+    cross_acc(vv, hf, fn);
+    cross_acc(vw, hf, ff);
+  }
+
+  // the bias torques: inverse dynamics at qdd = 0 with gravity and contact
   template <class R, class S>
-  TO_DEV static void rnea(const ParamsT<R>& P, const S* q, const S* qd, const S* qdd, bool grav, bool contact,
-                          S* tau) {
+  TO_DEV static void rnea(const ParamsT<R>& P, const S* q, const S* qd, S* tau) {
+    constexpr bool contact = KIND == RK_QUAD;
     S E[N][9], r[N][3], vw[N][3], vv[N][3], fn[N][3], ff[N][3];
-    S aw[3], av[3];
     S E0[KIND == RK_QUAD ? N : 1][9], p0[KIND == RK_QUAD ? N : 1][3];
     S awb[N][3], avb[N][3];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       joint_transform(P, i, q[i], E[i], r[i]);
-      const int pa = parent(i);
-      S pw[3], pv[3], paw[3], pav[3];
-      if (pa < 0) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          pw[k] = S(R(0)); pv[k] = S(R(0)); paw[k] = S(R(0));
-          pav[k] = grav ? S(-P.g[k]) : S(R(0));
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          pw[k] = vw[pa][k]; pv[k] = vv[pa][k]; paw[k] = awb[pa][k]; pav[k] = avb[pa][k];
-        }
-      }
-      // X m = (E w, E (v - r x w))
-      S t[3], rw[3];
-      cross(r[i], pw, rw);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) t[k] = pv[k] - rw[k];
-      jmv(jtype(i), E[i], pw, vw[i]);
-      jmv(jtype(i), E[i], t, vv[i]);
-      cross(r[i], paw, rw);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) t[k] = pav[k] - rw[k];
-      jmv(jtype(i), E[i], paw, aw);
-      jmv(jtype(i), E[i], t, av);
-      // joint motion S qd, S qdd; velocity-product term v x (S qd)
-      const int jt = jtype(i);
-      S sw[3] = {S(R(0)), S(R(0)), S(R(0))}, sv[3] = {S(R(0)), S(R(0)), S(R(0))};
-      if (jt <= 2) sw[jt] = qd[i]; else sv[jt - 3] = qd[i];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) { vw[i][k] = vw[i][k] + sw[k]; vv[i][k] = vv[i][k] + sv[k]; }
-      S c1[3], c2[3], c3[3];
-      cross(vw[i], sw, c1);
-      cross(vw[i], sv, c2);
-      cross(vv[i], sw, c3);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) { aw[k] = aw[k] + c1[k]; av[k] = av[k] + c2[k] + c3[k]; }
-      if (jt <= 2) aw[jt] = aw[jt] + qdd[i]; else av[jt - 3] = av[jt - 3] + qdd[i];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) { awb[i][k] = aw[k]; avb[i][k] = av[k]; }
-      // f = I a + v x* (I v)
-      S In[3], If[3], hn[3], hf[3];
-      inertia_mul(P, i, aw, av, In, If);
-      inertia_mul(P, i, vw[i], vv[i], hn, hf);
-      S x1[3], x2[3], x3[3];
-      cross(vw[i], hn, x1);
-      cross(vv[i], hf, x2);
-      cross(vw[i], hf, x3);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) { fn[i][k] = In[k] + x1[k] + x2[k]; ff[i][k] = If[k] + x3[k]; }
+      const int pa = parent(i), jt = jtype(i), pb = pa < 0 ? 0 : pa;
+      S Epw[3], Ept[3], hn[3], hf[3];
+      body_bias(P, i, E[i], r[i], qd[i], vw[pb], vv[pb], awb[pb], avb[pb], Epw, Ept, vw[i], vv[i], awb[i], avb[i], hn,
+                hf, fn[i], ff[i]);
       if (KIND == RK_QUAD) {
         if (pa < 0) {
 #pragma unroll
@@ -338,16 +404,16 @@ struct SysRigid {
 #pragma unroll
           for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int b = 0; b < 3; ++b)
-              E0[i][a * 3 + b] = E[i][a * 3 + 0] * E0[pa][b] + E[i][a * 3 + 1] * E0[pa][3 + b] + E[i][a * 3 + 2] * E0[pa][6 + b];
+            for (int b = 0; b < 3; ++b) E0[i][a * 3 + b] = e_row(jt, E[i], E0[pa], a, b);
           S wr[3];
           mtv(E0[pa], r[i], wr);
 #pragma unroll
           for (int k = 0; k < 3; ++k) p0[i][k] = p0[pa][k] + wr[k];
         }
       }
+      (void)jt;
     }
-    if (KIND == RK_QUAD && contact) {
+    if (contact) {
 #pragma unroll
       for (int ft = 0; ft < kFeet; ++ft) {
         const int bi = foot_body(ft);
@@ -412,6 +478,8 @@ struct SysRigid {
   // parallel-axis shift.  Bodies are ordered parents first.
   template <class R>
   TO_DEV static void mass_chol(const ParamsT<R>& P, const R* q, R* L) {
+    // the arm's float32 solves are chaotic and keep the full products' bits
+    constexpr bool kFull = KIND == RK_ARM7 && sizeof(R) == 4;
     R E[N][9], r[N][3];
     R cm[N], ch[N][3], cI[N][6];   // cI: xx, yy, zz, xy, xz, yz
 #pragma unroll
@@ -442,12 +510,15 @@ struct SysRigid {
 #pragma unroll
       for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) T[a * 3 + b] = I3[a * 3 + 0] * e[0 * 3 + b] + I3[a * 3 + 1] * e[1 * 3 + b] + I3[a * 3 + 2] * e[2 * 3 + b];
+        for (int b = 0; b < 3; ++b)
+          T[a * 3 + b] = kFull ? I3[a * 3 + 0] * e[0 * 3 + b] + I3[a * 3 + 1] * e[1 * 3 + b] + I3[a * 3 + 2] * e[2 * 3 + b]
+                               : e_col(jtype(i), I3, e, a, b);
       R IA[6];
       const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
       for (int k = 0; k < 6; ++k)
-        IA[k] = e[0 * 3 + ia[k]] * T[0 * 3 + ib[k]] + e[1 * 3 + ia[k]] * T[1 * 3 + ib[k]] + e[2 * 3 + ia[k]] * T[2 * 3 + ib[k]];
+        IA[k] = kFull ? e[0 * 3 + ia[k]] * T[0 * 3 + ib[k]] + e[1 * 3 + ia[k]] * T[1 * 3 + ib[k]] + e[2 * 3 + ia[k]] * T[2 * 3 + ib[k]]
+                      : et_row(jtype(i), e, T, ia[k], ib[k]);
       // shift to the parent origin (child origin at r):
       // I_O = I_A + m (|r|^2 1 - r r^T) + 2 (r.h_A) 1 - (h_A r^T + r h_A^T)
       const R r2 = rr[0] * rr[0] + rr[1] * rr[1] + rr[2] * rr[2];
@@ -564,10 +635,8 @@ struct SysRigid {
   // one substep's acceleration: qdd = M^{-1} (tau - h); also returns L
   template <class R>
   TO_DEV static void accel(const ParamsT<R>& P, const R* q, const R* qd, const R* tau, R* qdd, R* L) {
-    R z[N], h[N], rhs[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) z[i] = R(0);
-    rnea<R, R>(P, q, qd, z, true, KIND == RK_QUAD, h);
+    R h[N], rhs[N];
+    rnea<R, R>(P, q, qd, h);
     mass_chol(P, q, L);
 #pragma unroll
     for (int i = 0; i < N; ++i) rhs[i] = tau[i] - h[i];
@@ -643,10 +712,7 @@ struct SysRigid {
       g.sync();
       R hb[N];
       if (mine) {
-        R z[N];
-#pragma unroll
-        for (int i = 0; i < N; ++i) z[i] = R(0);
-        rnea<R, R>(P, xh, xh + N, z, true, KIND == RK_QUAD, hb);
+        rnea<R, R>(P, xh, xh + N, hb);
       } else if (c >= H && slot < kStepSlots && flag[slot] != R(0)) {
         mass_chol_mem(P, sq, sL);
       }
@@ -794,25 +860,12 @@ struct SysRigid {
     static constexpr int elems = prim > step ? prim : step;
   };
 
-  // y += a x b
-  template <class S> TO_DEV static void cross_acc(const S* a, const S* b, S* y) {
-    y[0] += a[1] * b[2] - a[2] * b[1];
-    y[1] += a[2] * b[0] - a[0] * b[2];
-    y[2] += a[0] * b[1] - a[1] * b[0];
-  }
   // y -= s (e_ax x z): the change of E x under dq about joint axis ax
   template <class S> TO_DEV static void rot_tangent(int ax, S s, const S* z, S* y) {
     if (ax == 0) { y[1] += s * z[2]; y[2] -= s * z[1]; }
     else if (ax == 1) { y[0] -= s * z[2]; y[2] += s * z[0]; }
     else { y[0] += s * z[1]; y[1] -= s * z[0]; }
   }
-  // e_ax x z
-  template <class S> TO_DEV static void axis_cross(int ax, const S* z, S* y) {
-    if (ax == 0) { y[0] = S(0); y[1] = -z[2]; y[2] = z[1]; }
-    else if (ax == 1) { y[0] = z[2]; y[1] = S(0); y[2] = -z[0]; }
-    else { y[0] = -z[1]; y[1] = z[0]; y[2] = S(0); }
-  }
-
   // A substep's primal for the derivative lanes comes in two halves around
   // the solve for qdd, so that the joint transforms, the velocities, the
   // world poses and the contact forces are evaluated once (the tangent pass
@@ -831,47 +884,17 @@ struct SysRigid {
       for (int k = 0; k < 9; ++k) pr.E[i][k] = E[k];
 #pragma unroll
       for (int k = 0; k < 3; ++k) pr.r[i][k] = r[k];
-      R pw[3], pv[3], paw[3], pav[3];
+      const int pb = pa < 0 ? 0 : pa;
+      R Epw[3], Ept[3], vw[3], vv[3], hn[3], hf[3], pw[3], pv[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) { pw[k] = pr.vw[pb][k]; pv[k] = pr.vv[pb][k]; }
+      body_bias(P, i, E, r, qd[i], pw, pv, aw[pb], av[pb], Epw, Ept, vw, vv, aw[i], av[i], hn, hf, fn[i], ff[i]);
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        pw[k] = pa < 0 ? R(0) : pr.vw[pa][k];
-        pv[k] = pa < 0 ? R(0) : pr.vv[pa][k];
-        paw[k] = pa < 0 ? R(0) : aw[pa][k];
-        pav[k] = pa < 0 ? -P.g[k] : av[pa][k];
-      }
-      R t[3], rw[3], Epw[3], Ept[3];
-      cross(r, pw, rw);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) t[k] = pv[k] - rw[k];
-      jmv(jt, E, pw, Epw);
-      jmv(jt, E, t, Ept);
-      R sw[3] = {R(0), R(0), R(0)}, sv[3] = {R(0), R(0), R(0)};
-      if (jt <= 2) sw[jt] = qd[i]; else sv[jt - 3] = qd[i];
-      R vw[3], vv[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        vw[k] = Epw[k] + sw[k];
-        vv[k] = Ept[k] + sv[k];
         pr.Epw[i][k] = Epw[k]; pr.Ept[i][k] = Ept[k];
         pr.vw[i][k] = vw[k]; pr.vv[i][k] = vv[k];
+        pr.hn[i][k] = hn[k]; pr.hf[i][k] = hf[k];
       }
-      // the acceleration at qdd = 0 and the body force it needs
-      cross(r, paw, rw);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) t[k] = pav[k] - rw[k];
-      jmv(jt, E, paw, aw[i]);
-      jmv(jt, E, t, av[i]);
-      cross_acc(vw, sw, aw[i]);
-      cross_acc(vw, sv, av[i]);
-      cross_acc(vv, sw, av[i]);
-      R In[3], If[3], hn[3], hf[3];
-      inertia_mul(P, i, aw[i], av[i], In, If);
-      inertia_mul(P, i, vw, vv, hn, hf);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) { pr.hn[i][k] = hn[k]; pr.hf[i][k] = hf[k]; fn[i][k] = In[k]; ff[i][k] = If[k]; }
-      cross_acc(vw, hn, fn[i]);
-      cross_acc(vv, hf, fn[i]);
-      cross_acc(vw, hf, ff[i]);
       if (KIND == RK_QUAD) {
         if (pa < 0) {
 #pragma unroll
@@ -882,8 +905,7 @@ struct SysRigid {
 #pragma unroll
           for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int b = 0; b < 3; ++b)
-              pr.E0[i][a * 3 + b] = E[a * 3 + 0] * pr.E0[pa][b] + E[a * 3 + 1] * pr.E0[pa][3 + b] + E[a * 3 + 2] * pr.E0[pa][6 + b];
+            for (int b = 0; b < 3; ++b) pr.E0[i][a * 3 + b] = e_row(jt, E, pr.E0[pa], a, b);
           R wr[3];
           mtv(pr.E0[pa], r, wr);
 #pragma unroll
@@ -954,29 +976,33 @@ struct SysRigid {
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int pa = parent(i), jt = jtype(i);
-      R paw[3], pav[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        paw[k] = pa < 0 ? R(0) : pr.aw[pa][k];
-        pav[k] = pa < 0 ? -P.g[k] : av[pa][k];
-      }
       const R* E = pr.E[i];
-      R t[3], rw[3], Epa[3], Epb[3], vw[3], vv[3], hn[3], hf[3];
+      const int ax = jt <= 2 ? jt : jt - 3;
+      R t[3], Epa[3], Epb[3], vw[3], vv[3], hn[3], hf[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) { vw[k] = pr.vw[i][k]; vv[k] = pr.vv[i][k]; hn[k] = pr.hn[i][k]; hf[k] = pr.hf[i][k]; }
-      cross(pr.r[i], paw, rw);
+      if (pa < 0) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) t[k] = pav[k] - rw[k];
-      jmv(jt, E, paw, Epa);
+        for (int k = 0; k < 3; ++k) { Epa[k] = R(0); t[k] = -P.g[k]; }
+      } else {
+        R paw[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { paw[k] = pr.aw[pa][k]; t[k] = av[pa][k]; }
+        cross_sub(pr.r[i], paw, t);
+        jmv(jt, E, paw, Epa);
+      }
       jmv(jt, E, t, Epb);
-      R sw[3] = {R(0), R(0), R(0)}, sv[3] = {R(0), R(0), R(0)};
-      if (jt <= 2) sw[jt] = pr.qd[i]; else sv[jt - 3] = pr.qd[i];
       R aw[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) { pr.Epa[i][k] = Epa[k]; pr.Epb[i][k] = Epb[k]; aw[k] = Epa[k]; av[i][k] = Epb[k]; }
-      cross_acc(vw, sw, aw);
-      cross_acc(vw, sv, av[i]);
-      cross_acc(vv, sw, av[i]);
+      if (pa >= 0) {
+        if (jt <= 2) {
+          axis_acc(vw, ax, pr.qd[i], aw);
+          axis_acc(vv, ax, pr.qd[i], av[i]);
+        } else {
+          axis_acc(vw, ax, pr.qd[i], av[i]);
+        }
+      }
       if (jt <= 2) aw[jt] += pr.qdd[i]; else av[i][jt - 3] += pr.qdd[i];
 #pragma unroll
       for (int k = 0; k < 3; ++k) pr.aw[i][k] = aw[k];
@@ -1033,50 +1059,49 @@ struct SysRigid {
       const int jt = jtype(i);
       const bool rev = jt <= 2;
       const int ax = rev ? jt : jt - 3;
-      const R sq = rev ? dq[i] : R(0);          // rotation tangent
       R dr[3] = {R(0), R(0), R(0)};
       if (!rev) dr[ax] = dq[i];
       const R* E = pr.E[i];
       const R* r = pr.r[i];
-      R dpw[3], dpv[3], dpaw[3], dpav[3], pw[3], paw[3];
-      for (int k = 0; k < 3; ++k) {
-        dpw[k] = pa < 0 ? R(0) : dvw[pa][k];
-        dpv[k] = pa < 0 ? R(0) : dvv[pa][k];
-        dpaw[k] = pa < 0 ? R(0) : daw[pa][k];
-        dpav[k] = pa < 0 ? R(0) : dav[pa][k];
-        pw[k] = pa < 0 ? R(0) : pr.vw[pa][k];
-        paw[k] = pa < 0 ? R(0) : pr.aw[pa][k];
+      R t[3];
+      if (pa < 0) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { dvw[i][k] = R(0); dvv[i][k] = R(0); daw[i][k] = R(0); dav[i][k] = R(0); }
+      } else {
+        R pw[3], paw[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { pw[k] = pr.vw[pa][k]; paw[k] = pr.aw[pa][k]; }
+        // velocity
+        jmv(jt, E, dvw[pa], dvw[i]);
+        if (rev) rot_tangent(ax, dq[i], pr.Epw[i], dvw[i]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) t[k] = dvv[pa][k];
+        cross_sub(r, dvw[pa], t);
+        if (!rev) axis_acc(pw, ax, dq[i], t);
+        jmv(jt, E, t, dvv[i]);
+        if (rev) rot_tangent(ax, dq[i], pr.Ept[i], dvv[i]);
+        // acceleration (qdd fixed)
+        jmv(jt, E, daw[pa], daw[i]);
+        if (rev) rot_tangent(ax, dq[i], pr.Epa[i], daw[i]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) t[k] = dav[pa][k];
+        cross_sub(r, daw[pa], t);
+        if (!rev) axis_acc(paw, ax, dq[i], t);
+        jmv(jt, E, t, dav[i]);
       }
-      // velocity
-      R t[3], u3[3];
-      jmv(jt, E, dpw, dvw[i]);
-      rot_tangent(ax, rev ? sq : R(0), pr.Epw[i], dvw[i]);
-      for (int k = 0; k < 3; ++k) t[k] = dpv[k];
-      cross(r, dpw, u3);
-      for (int k = 0; k < 3; ++k) t[k] -= u3[k];
-      cross(dr, pw, u3);
-      for (int k = 0; k < 3; ++k) t[k] -= u3[k];
-      jmv(jt, E, t, dvv[i]);
-      rot_tangent(ax, rev ? sq : R(0), pr.Ept[i], dvv[i]);
-      R sw[3] = {R(0), R(0), R(0)}, sv[3] = {R(0), R(0), R(0)}, dsw[3] = {R(0), R(0), R(0)}, dsv[3] = {R(0), R(0), R(0)};
-      if (rev) { sw[ax] = pr.qd[i]; dsw[ax] = dqd[i]; } else { sv[ax] = pr.qd[i]; dsv[ax] = dqd[i]; }
-      for (int k = 0; k < 3; ++k) { dvw[i][k] += dsw[k]; dvv[i][k] += dsv[k]; }
-      // acceleration (qdd fixed)
-      jmv(jt, E, dpaw, daw[i]);
-      rot_tangent(ax, rev ? sq : R(0), pr.Epa[i], daw[i]);
-      for (int k = 0; k < 3; ++k) t[k] = dpav[k];
-      cross(r, dpaw, u3);
-      for (int k = 0; k < 3; ++k) t[k] -= u3[k];
-      cross(dr, paw, u3);
-      for (int k = 0; k < 3; ++k) t[k] -= u3[k];
-      jmv(jt, E, t, dav[i]);
-      rot_tangent(ax, rev ? sq : R(0), pr.Epb[i], dav[i]);
-      cross_acc(dvw[i], sw, daw[i]);
-      cross_acc(pr.vw[i], dsw, daw[i]);
-      cross_acc(dvw[i], sv, dav[i]);
-      cross_acc(pr.vw[i], dsv, dav[i]);
-      cross_acc(dvv[i], sw, dav[i]);
-      cross_acc(pr.vv[i], dsw, dav[i]);
+      if (rev) rot_tangent(ax, dq[i], pr.Epb[i], dav[i]);
+      if (rev) dvw[i][ax] += dqd[i]; else dvv[i][ax] += dqd[i];
+      if (pa >= 0) {
+        if (rev) {
+          axis_acc(dvw[i], ax, pr.qd[i], daw[i]);
+          axis_acc(pr.vw[i], ax, dqd[i], daw[i]);
+          axis_acc(dvv[i], ax, pr.qd[i], dav[i]);
+          axis_acc(pr.vv[i], ax, dqd[i], dav[i]);
+        } else {
+          axis_acc(dvw[i], ax, pr.qd[i], dav[i]);
+          axis_acc(pr.vw[i], ax, dqd[i], dav[i]);
+        }
+      }
       // body force
       R dIn[3], dIf[3], dhn[3], dhf[3];
       inertia_mul(P, i, daw[i], dav[i], dIn, dIf);
@@ -1096,8 +1121,7 @@ struct SysRigid {
           for (int k = 0; k < 3; ++k) dp0[i][k] = dr[k];
         } else {
           for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b)
-              dE0[i][a * 3 + b] = E[a * 3 + 0] * dE0[pa][b] + E[a * 3 + 1] * dE0[pa][3 + b] + E[a * 3 + 2] * dE0[pa][6 + b];
+            for (int b = 0; b < 3; ++b) dE0[i][a * 3 + b] = e_row(jt, E, dE0[pa], a, b);
           R w1[3], w2[3];
           mtv(dE0[pa], r, w1);
           mtv(pr.E0[pa], dr, w2);
@@ -1108,7 +1132,7 @@ struct SysRigid {
           for (int b = 0; b < 3; ++b) {
             const R col[3] = {E0[0 * 3 + b], E0[1 * 3 + b], E0[2 * 3 + b]};
             R y[3] = {R(0), R(0), R(0)};
-            rot_tangent(ax, sq, col, y);
+            rot_tangent(ax, dq[i], col, y);
             for (int a = 0; a < 3; ++a) dE0[i][a * 3 + b] += y[a];
           }
         }
@@ -1158,20 +1182,19 @@ struct SysRigid {
       if (pa >= 0) {
         // d(E^T y) = E^T dy + dq E^T (e_ax x y) for a revolute joint
         const R* E = pr.E[i];
-        R yn[3], yf[3], den[3], def[3], w1[3];
+        R yn[3], yf[3], den[3], def[3];
         for (int k = 0; k < 3; ++k) { yn[k] = dfn[i][k]; yf[k] = dff[i][k]; }
         if (rev) {
-          axis_cross(ax, pr.fn[i], w1);
-          for (int k = 0; k < 3; ++k) yn[k] += dq[i] * w1[k];
-          axis_cross(ax, pr.ff[i], w1);
-          for (int k = 0; k < 3; ++k) yf[k] += dq[i] * w1[k];
+          rot_tangent(ax, -dq[i], pr.fn[i], yn);
+          rot_tangent(ax, -dq[i], pr.ff[i], yf);
         }
         jmtv(jt, E, yn, den);
         jmtv(jt, E, yf, def);
-        R ef[3], dr[3] = {R(0), R(0), R(0)};
-        if (!rev) dr[ax] = dq[i];
-        jmtv(jt, E, pr.ff[i], ef);
-        cross_acc(dr, ef, den);
+        if (!rev) {
+          R ef[3];
+          jmtv(jt, E, pr.ff[i], ef);
+          axis_acc(ef, ax, -dq[i], den);
+        }
         cross_acc(pr.r[i], def, den);
         for (int k = 0; k < 3; ++k) { dfn[pa][k] += den[k]; dff[pa][k] += def[k]; }
       }
