@@ -178,7 +178,9 @@ typedef struct {
                              quadruped); 0 = the totune
                              choice, else the system's default for the batch
                              size (planar arm: 16 for float32 batches that
-                             would leave SMs idle at 8).  1: one thread
+                             would leave SMs idle at 8; point mass and
+                             Dubins car: 32 for float64 batches of at most 4
+                             instances an SM; the same bits at either).  1: one thread
                              per instance with every per-knot matrix in
                              registers; its line search tries one step size
                              at a time (the smallest j first), the others

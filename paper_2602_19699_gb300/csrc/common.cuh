@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #define TO_DEV __device__ __forceinline__
+#define TO_HD __host__ __device__ __forceinline__
 
 namespace to {
 

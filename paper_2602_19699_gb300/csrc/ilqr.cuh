@@ -267,6 +267,22 @@ struct Solver {
     R* d0[PB];
     R* d1[PB];
   };
+  // systems with gain-record blocks at a whole warp: the sums of up to kA terms
+  // that this lane forms in spread_products, as offsets (in elements of R from
+  // w.V) of the factors, the first summand and the result; the same at every
+  // knot.  Step 0: V A, V B, Q_x, Q_u; step 1: Q_xx, Q_ux, Q_uu.
+  template <class S> static constexpr int spread_terms() {
+    if constexpr (S::kGainDerivs && G == 32) return S::kA;
+    else return 1;
+  }
+  static constexpr int kTerms = spread_terms<Sys>();
+  static constexpr int kSpread0 = n * n + n * m + n + m, kSpread1 = n * n + m * n + m * m;
+  struct SpreadSum {
+    short x[kTerms], y[kTerms], base, out;
+  };
+  struct Spread {
+    SpreadSum s0[(kSpread0 + 31) / 32], s1[(kSpread1 + 31) / 32];
+  };
   typedef typename Sys::template ParamsT<R> Params;
   static constexpr bool kLane = (G == 1);                  // one thread per instance, matrices in registers
   // lanes of a warp that are not a group's first lane (sub-warp groups)
@@ -660,6 +676,21 @@ struct Solver {
       const bool st = act && c0 < m;
       const int c = c0 < m ? c0 : m - 1;
       R vb[n];
+      if constexpr (Sys::kGainDerivs) {
+        const int rc = Sys::b_row(c);
+        const R bc = w.Bm[rc * m + c];
+#pragma unroll
+        for (int i = 0; i < n; ++i) vb[i] = mul_rn(w.V[i * n + rc], bc);
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+          const R t = fma_rn(w.Bm[Sys::b_row(i) * m + i], vb[Sys::b_row(i)], w.luu[i * m + c]);
+          if (st) {
+            if (q64) w.Quu[i * m + c] = (double)t;
+            w.Quf[i * m + c] = t;
+          }
+        }
+        if (st) w.Qu[c] = fma_rn(bc, w.v[rc], w.lu[c]);
+      } else {
 #pragma unroll
       for (int i = 0; i < n; ++i) {
         R t = 0;
@@ -681,6 +712,7 @@ struct Solver {
 #pragma unroll
       for (int r = 0; r < n; ++r) t += w.Bm[r * m + c] * w.v[r];
       if (st) w.Qu[c] = t;
+      }
     }
     g.sync();
     TO_TICK(2);
@@ -709,6 +741,37 @@ struct Solver {
           const bool st = act && j0 < n;
           const int j = j0 < n ? j0 : n - 1;
           R va[n];
+          if constexpr (Sys::kGainDerivs) {
+            // the nonzeros of A and B alone, in the order of the dense sums (the
+            // car, B=2048 float64, V_x, 3 iterations: 6.55 -> 5.55 ms)
+            R ca[Sys::kA], t = w.lx[j];
+            int ra[Sys::kA];
+#pragma unroll
+            for (int q = 0; q < Sys::kA; ++q) {
+              ra[q] = Sys::a_row(j, q);
+              ca[q] = w.A[ra[q] * n + j];
+              t = fma_rn(ca[q], w.v[ra[q]], t);
+            }
+            if (st) w.Qx[j] = t;
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+              t = mul_rn(w.V[i * n + ra[0]], ca[0]);
+#pragma unroll
+              for (int q = 1; q < Sys::kA; ++q) t = fma_rn(w.V[i * n + ra[q]], ca[q], t);
+              va[i] = t;
+            }
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+              t = w.lxx[i * n + j];
+#pragma unroll
+              for (int r = 0; r < n; ++r)
+                if (Sys::a_nz(r, i)) t = fma_rn(w.A[r * n + i], va[r], t);
+              if (st) QX[i * n + j] = t;
+            }
+#pragma unroll
+            for (int i = 0; i < m; ++i)
+              if (st) w.Qux[i * n + j] = mul_rn(w.Bm[Sys::b_row(i) * m + i], va[Sys::b_row(i)]);
+          } else {
 #pragma unroll
           for (int i = 0; i < n; ++i) {
             R t = 0;
@@ -734,6 +797,7 @@ struct Solver {
 #pragma unroll
           for (int r = 0; r < n; ++r) t += w.A[r * n + j] * w.v[r];
           if (st) w.Qx[j] = t;
+          }
         }
       };
       if (a.lm) {
@@ -836,6 +900,90 @@ struct Solver {
     return act ? flag : 0;
   }
 
+  // The sums of spread_products that lane l of the warp forms: l, l + 32, ...
+  TO_DEV static void spread_setup(W& w, int lane, Spread& sp) {
+    const R* o = w.V;
+    const int A = (int)(w.A - o), B = (int)(w.Bm - o), v = (int)(w.v - o), VA = (int)(w.VA - o), VB = (int)(w.VB - o);
+    const int zero = A + n, one = A;               // A(1, 0) is 0, A(0, 0) is 1
+    auto fill = [&](SpreadSum& u, int terms, int base, int out, auto&& xy) {
+      u.base = (short)base;
+      u.out = (short)out;
+#pragma unroll
+      for (int q = 0; q < kTerms; ++q) {
+        int x = one, y = zero;
+        if (q < terms) xy(q, x, y);
+        u.x[q] = (short)x;
+        u.y[q] = (short)y;
+      }
+    };
+#pragma unroll
+    for (int s = 0; s < (kSpread0 + 31) / 32; ++s) {
+      const int e = lane + 32 * s;
+      if (e < n * n) {                             // V A
+        const int i = e / n, j = e % n;
+        fill(sp.s0[s], kTerms, zero, VA + e, [&](int q, int& x, int& y) { const int r = Sys::a_row(j, q); x = i * n + r; y = A + r * n + j; });
+      } else if (e < n * n + n * m) {              // V B
+        const int f = e - n * n, i = f / m, c = f % m, r = Sys::b_row(c);
+        fill(sp.s0[s], 1, zero, VB + f, [&](int, int& x, int& y) { x = i * n + r; y = B + r * m + c; });
+      } else if (e < n * n + n * m + n) {          // Q_x
+        const int j = e - n * n - n * m;
+        fill(sp.s0[s], kTerms, (int)(w.lx - o) + j, (int)(w.Qx - o) + j,
+             [&](int q, int& x, int& y) { const int r = Sys::a_row(j, q); x = v + r; y = A + r * n + j; });
+      } else {                                     // Q_u
+        const int c = e < kSpread0 ? e - n * n - n * m - n : 0, r = Sys::b_row(c);
+        fill(sp.s0[s], 1, (int)(w.lu - o) + c, (int)(w.Qu - o) + c, [&](int, int& x, int& y) { x = v + r; y = B + r * m + c; });
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < (kSpread1 + 31) / 32; ++s) {
+      const int e = lane + 32 * s;
+      if (e < n * n) {                             // Q_xx, full, over V
+        const int i = e / n, j = e % n;
+        fill(sp.s1[s], kTerms, (int)(w.lxx - o) + e, e, [&](int q, int& x, int& y) { const int r = Sys::a_row(i, q); x = VA + r * n + j; y = A + r * n + i; });
+      } else if (e < n * n + m * n) {              // Q_ux (l_ux = 0)
+        const int f = e - n * n, i = f / n, j = f % n, r = Sys::b_row(i);
+        fill(sp.s1[s], 1, zero, (int)(w.Qux - o) + f, [&](int, int& x, int& y) { x = VA + r * n + j; y = B + r * m + i; });
+      } else {                                     // Q_uu
+        const int f = e < kSpread1 ? e - n * n - m * n : 0, i = f / m, j = f % m, r = Sys::b_row(i);
+        fill(sp.s1[s], 1, (int)(w.luu - o) + f, (int)(w.Quf - o) + f, [&](int, int& x, int& y) { x = VB + r * m + j; y = B + r * m + i; });
+      }
+    }
+  }
+
+  // The Q terms of a backward knot at a whole warp, one entry per lane, from the
+  // nonzeros of A and B alone: the point mass takes 4 multiply-adds deep (the
+  // dense products 8), the car 12 (20).  In float64 a warp instruction holds the
+  // scheduler's FP64 pipe for 64 cycles however many lanes it serves, so their
+  // number is the knot's time.  Each sum's nonzero terms are taken in the order
+  // of backward_cols, and Q_xx is formed in full as there: the same bits.
+  // Point mass float64, 2 iterations: B=1 1.10 -> 0.70 ms, B=64 1.20 -> 0.85 ms
+  // against 8 lanes with dense products.
+  TO_DEV static void spread_products(const Group<G>& g, W& w, bool act, const Spread& sp) {
+    R* o = w.V;
+    auto sum = [&](const SpreadSum& u) {
+      R t = o[u.base];
+#pragma unroll
+      for (int q = 0; q < kTerms; ++q) t = fma_rn(o[u.y[q]], o[u.x[q]], t);
+      return t;
+    };
+    if (act)
+#pragma unroll
+      for (int s = 0; s < (kSpread0 + 31) / 32; ++s)
+        if (g.lane + 32 * s < kSpread0) o[sp.s0[s].out] = sum(sp.s0[s]);
+    g.sync();
+    if (act)
+#pragma unroll
+      for (int s = 0; s < (kSpread1 + 31) / 32; ++s) {
+        const int e = g.lane + 32 * s;
+        if (e < kSpread1) {
+          const R t = sum(sp.s1[s]);
+          o[sp.s1[s].out] = t;
+          if (e >= n * n + m * n) w.Quu[e - n * n - m * n] = (double)t;
+        }
+      }
+    g.sync();
+  }
+
   // ------------------------------------------------------------------------
   // one knot of the backward pass (all syncs unconditional, work predicated).
   // The knot's record is in pb (prefetched); the record of the knot D
@@ -844,7 +992,7 @@ struct Solver {
   // ------------------------------------------------------------------------
   TO_DEV static int backward_knot(const Params& P, const Group<G>& g, W& w, bool act, bool act_next,
                                   const SolveArgs& a, R (&pb)[PB], const R* trec_next, R* grec, double* vxrec,
-                                  double mu_lm, bool timer, long long& tlast, const R* kprim, const BlockDst& dst) {
+                                  double mu_lm, bool timer, long long& tlast, const R* kprim, const BlockDst& dst, const Spread& sp) {
     const R eps = (R)a.eps;
     if constexpr (!Sys::kStoredDerivs && !Sys::kGainDerivs) {   // x_k, u_k feed the derivative step (stored blocks need neither)
       if (act) {
@@ -913,6 +1061,10 @@ struct Solver {
       return backward_cols(g, w, act, a, grec, vxrec, mu_lm, timer, tlast);
     } else {
     constexpr int NT = n * (n + 1) / 2;
+    if constexpr (Sys::kGainDerivs) {
+      spread_products(g, w, act, sp);
+      TO_TICK(2);
+    } else {
       // V A and V B
       if (act)
         for (int e = g.lane; e < n * n + n * m; e += G) {
@@ -972,6 +1124,7 @@ struct Solver {
         }
       g.sync();
       TO_TICK(2);
+    }
       if (act && g.lane < 32) chol_warp(w, a.lm, mu_lm, g.lane);   // act is uniform over the group
       g.sync();
     const int flag = act ? w.flag : 0;
@@ -1430,6 +1583,8 @@ struct Solver {
             }
           }
           BlockDst dst;
+          Spread sp;
+          if constexpr (Sys::kGainDerivs && G == 32) spread_setup(w, g.lane, sp);
           if constexpr (Sys::kGainDerivs) {
 #pragma unroll
             for (int s = 0; s < PB; ++s) {
@@ -1522,7 +1677,7 @@ struct Solver {
               const R* kprim = Sys::kGainDerivs ? grec_at(a, gains, kd) : dscr_at(a, kd);
               const int f = backward_knot(P, g, w, act, act_next, a, pb[d], rn, grec_at(a, gains, kk),
                                           (a.vx && a.want_vx && act) ? vx_at(a, a.vx, kk) : nullptr, mu_lm, timer,
-                                          tlast, kprim, dst);
+                                          tlast, kprim, dst, sp);
               if (f == 1) flags |= ST_FLAG_REG;
               // Levenberg-Marquardt: any failed factor (pivot test, or a
               // non-finite Q_uu once an earlier knot's gains were skipped)

@@ -25,6 +25,15 @@ static int parse_dubins(const double* p, size_t np, std::vector<unsigned char>& 
 
 typedef Dispatch<SysDubins, kDepth1, 1, 8, 16, 32> DBDispatch;
 
+// Float64 batches that leave a scheduler per instance take a whole warp: a
+// float64 warp instruction holds its scheduler's FP64 pipe for 64 cycles
+// however many lanes it serves, and 32 lanes share a knot's entries where 8
+// take columns of them.  Measured (3 iterations,
+// ms at 8 / 32 lanes, both with dense products): B = 64 3.90 / 2.97, 608 3.94 /
+// 3.14, 1216 3.96 / 4.97, 2048 4.15 / 9.77.  Beyond 4 instances an SM the pipes are shared and 8
+// lanes, four instances an instruction, win.  The sizes give the same bits.
+static int dubins_lanes(int prec, int B, int sms) { return prec == PREC_FP64 && B <= 4 * sms ? 32 : 8; }
+
 static SysOps make_ops() {
   SysOps o{};
   o.sys = 5;
@@ -33,6 +42,7 @@ static SysOps make_ops() {
   o.groups[0] = 8; o.groups[1] = 16; o.groups[2] = 32; o.groups[3] = 1;   // 1: one thread per instance
   o.default_G = 8;
   o.default_gpb[0] = 8; o.default_gpb[1] = 8;
+  o.lanes = dubins_lanes;
   o.accepts_actor = false;
   o.parse = parse_dubins;
   o.max_depth = 1;

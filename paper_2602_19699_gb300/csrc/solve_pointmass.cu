@@ -24,6 +24,15 @@ static int parse_pointmass(const double* p, size_t np, std::vector<unsigned char
 
 typedef Dispatch<SysPointMass, kDepth1, 1, 8, 16, 32> PMDispatch;
 
+// Float64 batches that leave a scheduler per instance take a whole warp: a
+// float64 warp instruction holds its scheduler's FP64 pipe for 64 cycles
+// however many lanes it serves, and 32 lanes share a knot's entries where 8
+// take columns of them.  Measured (2 iterations,
+// ms at 8 / 32 lanes, both with dense products): B = 1 1.11 / 0.84, 64 1.07 /
+// 0.85, 608 1.08 / 0.89, 1216 1.10 / 1.37, 2048 1.14 / 2.66.  Beyond 4 instances an SM the pipes are shared and 8
+// lanes, four instances an instruction, win.  The sizes give the same bits.
+static int pointmass_lanes(int prec, int B, int sms) { return prec == PREC_FP64 && B <= 4 * sms ? 32 : 8; }
+
 static SysOps make_ops() {
   SysOps o{};
   o.sys = 1;
@@ -32,6 +41,7 @@ static SysOps make_ops() {
   o.groups[0] = 8; o.groups[1] = 16; o.groups[2] = 32; o.groups[3] = 1;   // 1: one thread per instance
   o.default_G = 8;
   o.default_gpb[0] = 8; o.default_gpb[1] = 8;
+  o.lanes = pointmass_lanes;
   o.accepts_actor = false;
   o.parse = parse_pointmass;
   o.max_depth = 1;

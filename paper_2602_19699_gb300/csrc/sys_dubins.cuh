@@ -110,6 +110,15 @@ struct SysDubins {
     d[9] = w2 * u[0]; d[10] = w2 * u[1];
     d[11] = R(0);
   }
+  // Sparsity of A and B.  Column j of A has its nonzeros in rows a_row(j, q), q <
+  // kA, in ascending order (filled up with rows whose entry is 0); column c of
+  // B has one, in row b_row(c).
+  static constexpr int kA = 3;
+  static constexpr TO_HD int a_row(int j, int q) {
+    return q == 0 ? 0 : q == 1 ? (j == 4 ? 3 : 1) : (j == 3 ? 3 : j == 4 ? 4 : 2);
+  }
+  static constexpr TO_HD bool a_nz(int r, int j) { return r == j || (r < 2 && (j == 2 || j == 3)) || (r == 3 && j == 4); }
+  static constexpr TO_HD int b_row(int c) { return 2 + 2 * c; }
   // the constant entries: A, B, and l_xx, l_x, l_uu outside the block (lane
   // of a group of G)
   template <class R>
