@@ -63,6 +63,7 @@ struct SysPlanar3 {
   // per lane (derivs_lane), and stored: A, B, l_xx, l_x, l_uu, l_u
   static constexpr bool kStoredDerivs = true;
   static constexpr bool kGainDerivs = false;
+  static constexpr bool kDeferCost = false;   // the cost shares the step's kinematics
   static constexpr int kDerivStride = n * n + n * m + n * n + n + m * m + m;
 
   // absolute link angles, link and centre-of-mass vectors, joint positions
@@ -249,7 +250,7 @@ struct SysPlanar3 {
     Kin<R> k;
     kinematics(P, xh, k);
     R l = P.wtau * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    each_bump(P.bc, P.nb, k.P[3][0], k.P[3][1], P.inv1, [&](R, R, R e) { l += P.bamp * e; });
+    each_bump<2>(P.bc, P.nb, k.P[3][0], k.P[3][1], P.inv1, [&](R, R, R e) { l += P.bamp * e; });
     R qdd[3], L[9];
     forward_dynamics(P, k, xh + 3, u, qdd, L);
     semi_implicit2<R, 3>(xh, xl, xh + 3, xl + 3, qdd, P.dt);
@@ -303,7 +304,7 @@ struct SysPlanar3 {
     Kin<R> k;
     kinematics(P, x, k);
     R l = P.wtau * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    each_bump(P.bc, P.nb, k.P[3][0], k.P[3][1], P.inv2, [&](R, R, R e) { l += P.bamp * e; });
+    each_bump<2>(P.bc, P.nb, k.P[3][0], k.P[3][1], P.inv2, [&](R, R, R e) { l += P.bamp * e; });
     return l;
   }
 
@@ -322,7 +323,7 @@ struct SysPlanar3 {
     ee_derivs(k, ee, J);
     R gee[2] = {0, 0}, H[2][2] = {{0, 0}, {0, 0}};
     const R is2 = P.is2;
-    each_bump(P.bc, P.nb, ee[0], ee[1], P.inv, [&](R d0, R d1, R ex) {
+    each_bump<2>(P.bc, P.nb, ee[0], ee[1], P.inv, [&](R d0, R d1, R ex) {
       const R e = P.bamp * ex;
       const R g0 = d0 * is2, g1 = d1 * is2;     // gradient of the exponent / -1
       gee[0] -= e * g0;
