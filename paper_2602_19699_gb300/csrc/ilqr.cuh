@@ -283,6 +283,8 @@ struct Solver {
   struct Spread {
     SpreadSum s0[(kSpread0 + 31) / 32], s1[(kSpread1 + 31) / 32];
   };
+  // running costs evaluated after a rollout by all of the group's lanes
+  static constexpr bool kDefer = Sys::kDeferCost && sizeof(R) == 8 && G > 1;
   typedef typename Sys::template ParamsT<R> Params;
   static constexpr bool kLane = (G == 1);                  // one thread per instance, matrices in registers
   // lanes of a warp that are not a group's first lane (sub-warp groups)
@@ -1430,6 +1432,37 @@ struct Solver {
     return reinterpret_cast<R*>(a.dscr) + ck(a, kn, a.knots_cap, CK_DSCR) * a.kscr;
   }
 
+  // The running costs of nc rolled-out candidates (slots written, the warp
+  // synchronised), G / nc knots at a time: lane f nc + c evaluates knot k0 + f of
+  // candidate c, and the costs are added up in the order of the knots, as a
+  // rollout that costs every knot on its way does.  In float64 an instruction
+  // holds the scheduler's FP64 pipe for 64 cycles however many lanes it serves;
+  // the three exponentials are 51 of the point mass's ~98 a knot.  Point mass
+  // float64, 2 iterations: B=1 0.70 -> 0.49 ms, B=64 0.85 -> 0.62 ms.
+  TO_DEV static void deferred_costs(const Params& P, const Group<G>& g, const SolveArgs& a, R* traj, long long base, int T,
+                                    int cur, bool fresh, bool on, int nc, Acc<R>& Jc) {
+    const int c = g.lane % nc, f = g.lane / nc, F = on ? G / nc : 0, first = (int)(threadIdx.x & 31) - g.lane;
+    const int slot = fresh ? 0 : (c < cur ? c : c + 1);
+    const int rounds = g.uniform_max(on ? (T + F - 1) / F : 0, nullptr), Fmax = g.uniform_max(F, nullptr);
+    for (int r = 0; r < rounds; ++r) {
+      const int k = r * F + f;
+      R l = R(0);
+      if (on && k < T) {
+        const R* q = rec(a, traj, base, k, slot);
+        R x[n], u[m];
+#pragma unroll
+        for (int i = 0; i < n; ++i) x[i] = q[i];
+#pragma unroll
+        for (int i = 0; i < m; ++i) u[i] = q[n + i];
+        l = Sys::running_cost(P, x, u);
+      }
+      for (int h = 0; h < Fmax; ++h) {
+        const R v = __shfl_sync(0xffffffffu, l, first + (h < F ? h * nc + c : g.lane));
+        if (h < F && r * F + h < T) Jc.add(v);
+      }
+    }
+  }
+
   // ------------------------------------------------------------------------
   // the kernel body
   // ------------------------------------------------------------------------
@@ -1757,6 +1790,9 @@ struct Solver {
                 if (d < T) prefetch_fwd(g, pf[d], rec(a, traj, base, d, cur), grec_at(a, gains, base + d));
             }
           }
+          // the lanes that roll out (one, or LW) are a fraction of the group:
+          // the others share the running costs after the rollout
+          const bool defer = kDefer && need && (single || LW < G);
           const int kr = g.uniform_max(need ? T : 0, &w.sel);
           for (int k0 = 0; k0 < kr; k0 += D) {
 #pragma unroll
@@ -1814,7 +1850,12 @@ struct Solver {
               }
               // the padding too: whole 32-byte sectors reach L2 without a read
               put_record(rec(a, traj, base, k, slot), xh, uh, xlo);
-              if constexpr (!Sys::template kGroupStep<G>) Jc.add(Sys::cost_step2(P, xh, xlo, uh));
+              if constexpr (kDefer) {
+                if (defer) Sys::step2(P, xh, xlo, uh);
+                else Jc.add(Sys::cost_step2(P, xh, xlo, uh));
+              } else if constexpr (!Sys::template kGroupStep<G>) {
+                Jc.add(Sys::cost_step2(P, xh, xlo, uh));
+              }
             }
             if constexpr (Sys::template kGroupStep<G>) {
               // the system's step is shared by partner lanes (group barriers inside;
@@ -1824,6 +1865,9 @@ struct Solver {
             }
             if constexpr (!kLane) g.sync();
           }
+          }
+          if constexpr (kDefer) {
+            if (!g.uniform_all(!defer)) deferred_costs(P, g, a, traj, base, T, cur, mode == M_NEW, defer, single ? 1 : LW, Jc);
           }
           double Jt = 0;
           int best = 0x7fffffff;

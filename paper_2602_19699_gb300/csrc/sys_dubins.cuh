@@ -58,6 +58,14 @@ struct SysDubins {
   template <class R>
   TO_DEV static R cost_step2(const ParamsT<R>& P, R* xh, R* xl, const R* u) {
     const R l = running_cost(P, xh, u);
+    step2(P, xh, xl, u);
+    return l;
+  }
+  // the next state alone: the running cost (three exponentials) is off the
+  // rollout's chain
+  static constexpr bool kDeferCost = true;
+  template <class R>
+  TO_DEV static void step2(const ParamsT<R>& P, R* xh, R* xl, const R* u) {
     R s, c;
     sincos(xh[2], &s, &c);
     const R v = xh[3] + xl[3];
@@ -67,7 +75,6 @@ struct SysDubins {
     acc2(xh[2], xl[2], P.dt * u[0]);
     acc2(xh[3], xl[3], dv);
     acc2(xh[4], xl[4], P.dt * u[1]);
-    return l;
   }
 
   template <class R>

@@ -54,12 +54,19 @@ struct SysPointMass {
   template <class R>
   TO_DEV static R cost_step2(const ParamsT<R>& P, R* xh, R* xl, const R* u) {
     const R l = running_cost(P, xh, u);
+    step2(P, xh, xl, u);
+    return l;
+  }
+  // the next state alone: the running cost (three exponentials) is off the
+  // rollout's chain
+  static constexpr bool kDeferCost = true;
+  template <class R>
+  TO_DEV static void step2(const ParamsT<R>& P, R* xh, R* xl, const R* u) {
     const R dpx = P.dt * xh[2] + P.dt * xl[2], dpy = P.dt * xh[3] + P.dt * xl[3];
     acc2(xh[0], xl[0], dpx);
     acc2(xh[1], xl[1], dpy);
     acc2(xh[2], xl[2], P.dt * u[0]);
     acc2(xh[3], xl[3], P.dt * u[1]);
-    return l;
   }
 
   template <class R>

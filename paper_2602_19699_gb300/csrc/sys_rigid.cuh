@@ -839,6 +839,7 @@ struct SysRigid {
   static constexpr bool kKnotParallel = true;
   static constexpr bool kStoredDerivs = false;
   static constexpr bool kGainDerivs = false;
+  static constexpr bool kDeferCost = false;
   // elements per stored substep primal (a whole number of 16-byte chunks)
   template <class R> static constexpr int kPrimStride = (int)(((sizeof(Prim<R>) + 15) / 16 * 16) / sizeof(R));
 
