@@ -451,24 +451,23 @@ TO_DEV void eigclip_small(R* Q, R eps) {
     }
 }
 
-// The same clip for larger blocks with runtime loops (small code; the
-// matrices live in local memory).  One thread.
+// The same clip of a larger block by the 32 lanes of a warp: Q (P x P, shared
+// memory) in place, W scratch of the same size; on is uniform over the warp, and
+// the barriers are taken either way.  The scalars of a rotation are formed on
+// every lane, its rows and columns by lane k for entry k.
 template <class R, int P>
-TO_DEV void eigclip_jacobi(R* Q, R eps) {
+TO_DEV void eigclip_warp(R* Q, R* W, R eps, int lane, bool on) {
+  static_assert(P <= 32, "a lane per row");
   R gmax = -R(1e30);
-  for (int i = 0; i < P; ++i) {
-    R s = Q[i * P + i];
-    for (int j = 0; j < P; ++j)
-      if (j != i) s += fabs(Q[i * P + j]);
-    gmax = s > gmax ? s : gmax;
-  }
-  if (gmax <= eps) {
-    for (int i = 0; i < P * P; ++i) Q[i] = (i % (P + 1) == 0) ? eps : R(0);
-    return;
-  }
-  R A[P * P], W[P * P];
-  {
-    bool pd = true;
+  bool pd = true;
+  if (on) {
+    for (int i = 0; i < P; ++i) {
+      R s = Q[i * P + i];
+      for (int j = 0; j < P; ++j)
+        if (j != i) s += fabs(Q[i * P + j]);
+      gmax = s > gmax ? s : gmax;
+    }
+    R A[P * P];
     for (int j = 0; j < P && pd; ++j) {
       R s = Q[j * P + j] - eps;
       for (int k = 0; k < j; ++k) s -= A[j * P + k] * A[j * P + k];
@@ -481,51 +480,70 @@ TO_DEV void eigclip_jacobi(R* Q, R eps) {
         A[i * P + j] = t * r;
       }
     }
-    if (pd) return;
   }
-  for (int i = 0; i < P * P; ++i) { A[i] = Q[i]; W[i] = (i % (P + 1) == 0) ? R(1) : R(0); }
+  __syncwarp();
+  if (!on) return;
+  if (gmax <= eps) {
+    for (int i = lane; i < P * P; i += 32) Q[i] = (i % (P + 1) == 0) ? eps : R(0);
+    __syncwarp();
+    return;
+  }
+  if (pd) return;
+  for (int i = lane; i < P * P; i += 32) W[i] = (i % (P + 1) == 0) ? R(1) : R(0);
+  __syncwarp();
   for (int sweep = 0; sweep < 30; ++sweep) {
     R off = 0, tot = 0;
     for (int p = 0; p < P; ++p)
       for (int q = 0; q < P; ++q) {
-        tot += A[p * P + q] * A[p * P + q];
-        if (p != q) off += A[p * P + q] * A[p * P + q];
+        tot += Q[p * P + q] * Q[p * P + q];
+        if (p != q) off += Q[p * P + q] * Q[p * P + q];
       }
     if (!(off > R(sizeof(R) == 4 ? 1e-14 : 1e-30) * tot)) break;
     for (int p = 0; p < P; ++p)
       for (int q = p + 1; q < P; ++q) {
-        const R apq = A[p * P + q];
+        const R apq = Q[p * P + q];
         if (apq == R(0)) continue;
-        const R tau = (A[q * P + q] - A[p * P + p]) / (R(2) * apq);
+        const R tau = (Q[q * P + q] - Q[p * P + p]) / (R(2) * apq);
         const R t = (tau >= R(0) ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
         const R c = rsqrt_(R(1) + t * t), s = t * c;
-        for (int k = 0; k < P; ++k) {
-          const R akp = A[k * P + p], akq = A[k * P + q];
-          A[k * P + p] = c * akp - s * akq;
-          A[k * P + q] = s * akp + c * akq;
+        __syncwarp();                    // every lane has read the pivot
+        if (lane < P) {
+          const R akp = Q[lane * P + p], akq = Q[lane * P + q];
+          Q[lane * P + p] = c * akp - s * akq;
+          Q[lane * P + q] = s * akp + c * akq;
         }
-        for (int k = 0; k < P; ++k) {
-          const R apk = A[p * P + k], aqk = A[q * P + k];
-          A[p * P + k] = c * apk - s * aqk;
-          A[q * P + k] = s * apk + c * aqk;
+        __syncwarp();
+        if (lane < P) {
+          const R apk = Q[p * P + lane], aqk = Q[q * P + lane];
+          Q[p * P + lane] = c * apk - s * aqk;
+          Q[q * P + lane] = s * apk + c * aqk;
+          const R wkp = W[lane * P + p], wkq = W[lane * P + q];
+          W[lane * P + p] = c * wkp - s * wkq;
+          W[lane * P + q] = s * wkp + c * wkq;
         }
-        for (int k = 0; k < P; ++k) {
-          const R wkp = W[k * P + p], wkq = W[k * P + q];
-          W[k * P + p] = c * wkp - s * wkq;
-          W[k * P + q] = s * wkp + c * wkq;
-        }
+        __syncwarp();
       }
   }
-  for (int i = 0; i < P; ++i)
-    for (int j = i; j < P; ++j) {
-      R s = 0;
+  // Q' = W diag(max(lambda, eps)) W^T, the entries kept in registers until
+  // every lane has read the diagonal
+  constexpr int kS = (P * P + 31) / 32;
+  R o[kS];
+#pragma unroll
+  for (int u = 0; u < kS; ++u) {
+    const int e = lane + 32 * u, i0 = e / P, j0 = e % P, i = i0 < j0 ? i0 : j0, j = i0 < j0 ? j0 : i0;
+    R s = 0;
+    if (e < P * P)
       for (int k = 0; k < P; ++k) {
-        const R d = A[k * P + k] > eps ? A[k * P + k] : eps;
+        const R d = Q[k * P + k] > eps ? Q[k * P + k] : eps;
         s += W[i * P + k] * d * W[j * P + k];
       }
-      Q[i * P + j] = s;
-      Q[j * P + i] = s;
-    }
+    o[u] = s;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < kS; ++u)
+    if (lane + 32 * u < P * P) Q[lane + 32 * u] = o[u];
+  __syncwarp();
 }
 
 }  // namespace to

@@ -1591,6 +1591,7 @@ struct Solver {
               if (d == sl) f(pb[d]);
           };
           if (bw) {
+            if constexpr (!Sys::kKnotParallel)
             if (g.lane == 0) {
               const R* r = rec(a, traj, base, T, cur);
               R xT[n];
@@ -1665,6 +1666,10 @@ struct Solver {
             }
           }
           if constexpr (Sys::kKnotParallel) {
+            Sys::template terminal_group<R, G>(P, g, bw, rec(a, traj, base, bw ? T : 0, cur), (R)a.eps, w.V, w.v, w.VA);
+            g.sync();
+            if (bw && a.vx && a.want_vx)
+              for (int i = g.lane; i < n; i += G) vx_at(a, a.vx, base + T)[i] = (double)w.v[i];
             // every lane: the substep primal chains of its knots (bw is uniform over a group of whole warps)
             if (bw)
               for (int k = g.lane; k < T; k += G) {

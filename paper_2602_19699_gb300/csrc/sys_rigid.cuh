@@ -768,46 +768,66 @@ struct SysRigid {
     (void)dq;
   }
 
-  // terminal-cost derivatives; the arm's end-effector term through forward
-  // kinematics: gradient and exact Hessian by nested dual numbers (one lane),
-  // then the q-block is eigen-clipped
-  template <class R>
-  TO_DEV static void terminal_derivs(const ParamsT<R>& P, const R* x, R eps, R* lxx, R* lx) {
-    for (int i = 0; i < n * n; ++i) lxx[i] = 0;
-    for (int i = 0; i < n; ++i) lx[i] = 0;
-    if (KIND == RK_ARM7) {
-      typedef Dl<Dl<R>> H;
-      R Q[N * N];
-      for (int a = 0; a < N; ++a)
-        for (int b = a; b < N; ++b) {
-          H q[N];
+  // Terminal-cost derivatives (V and v in shared memory), by a group of whole
+  // warps; on is uniform over it.  The arm's end-effector term goes through
+  // forward kinematics: gradient and exact Hessian by nested dual numbers, one
+  // pair of joints per lane, then the q-block is eigen-clipped by the lanes
+  // together (scratch: 2 N^2 elements).  On one lane, as it was, the 28 pairs and
+  // the Jacobi sweeps were a third of a solve: 7-DoF arm B=304 float64, T 10..20,
+  // 2 iterations, V_x 15.3 -> 9.0 ms; B=2048 float32, T 50..200, 2 iterations
+  // 27.5 -> 17.2 ms (the same bits; the kernel's code also shrank from 582 to 343
+  // KB).
+  template <class R, int G>
+  TO_DEV static void terminal_group(const ParamsT<R>& P, const Group<G>& g, bool on, const R* x, R eps, R* lxx, R* lx,
+                                    R* scratch) {
+    if (on) {
+      for (int e = g.lane; e < n * n; e += G) lxx[e] = R(0);
+      for (int e = g.lane; e < n; e += G) lx[e] = R(0);
+    }
+    g.sync();
+    if constexpr (KIND == RK_ARM7) {
+      static_assert(G == 32 && N * (N + 1) / 2 <= G, "a lane per pair of joints");
+      R* A = scratch;
+      if (on && g.lane < N * (N + 1) / 2) {
+        typedef Dl<Dl<R>> H;
+        int a = 0, b = g.lane;                        // pair (a, b), a <= b
+        while (b >= N - a) { b -= N - a; ++a; }
+        b += a;
+        H q[N];
 #pragma unroll
-          for (int k = 0; k < N; ++k) q[k] = H(Dl<R>(x[k], k == a ? R(1) : R(0)), Dl<R>(k == b ? R(1) : R(0), R(0)));
-          H ee[3];
-          ee_world(P, q, ee);
-          H l(Dl<R>(R(0)));
-          const H wee(Dl<R>(P.wee));
-          for (int k = 0; k < 3; ++k) {
-            const H d = ee[k] - H(Dl<R>(P.tgt[k]));
-            l = l + wee * (d * d);
-          }
-          Q[a * N + b] = l.d.d;
-          Q[b * N + a] = l.d.d;
-          if (a == b) lx[a] = l.v.d;
+        for (int k = 0; k < N; ++k) q[k] = H(Dl<R>(x[k], k == a ? R(1) : R(0)), Dl<R>(k == b ? R(1) : R(0), R(0)));
+        H ee[3];
+        ee_world(P, q, ee);
+        H l(Dl<R>(R(0)));
+        const H wee(Dl<R>(P.wee));
+        for (int k = 0; k < 3; ++k) {
+          const H d = ee[k] - H(Dl<R>(P.tgt[k]));
+          l = l + wee * (d * d);
         }
-      eigclip_jacobi<R, N>(Q, eps);
-      for (int a = 0; a < N; ++a)
-        for (int b = 0; b < N; ++b) lxx[a * n + b] = Q[a * N + b];
-      const R v2 = R(2) * P.wvT;
-#pragma unroll
-      for (int j = 0; j < N; ++j) { lx[N + j] = v2 * x[N + j]; lxx[(N + j) * n + N + j] = v2 > eps ? v2 : eps; }
-    } else {
+        A[a * N + b] = l.d.d;
+        A[b * N + a] = l.d.d;
+        if (a == b) lx[a] = l.v.d;
+      }
+      g.sync();
+      eigclip_warp<R, N>(A, A + N * N, eps, g.lane, on);
+      if (on) {
+        for (int e = g.lane; e < N * N; e += G) lxx[(e / N) * n + e % N] = A[e];
+        const R v2 = R(2) * P.wvT;
+        if (g.lane < N) {
+          lx[N + g.lane] = v2 * x[N + g.lane];
+          lxx[(N + g.lane) * n + N + g.lane] = v2 > eps ? v2 : eps;
+        }
+      }
+    } else if (on) {
       const R s = P.tscale;
       const R z2 = R(2) * P.wz * s, r2 = R(2) * P.wrpy * s, x2 = R(2) * P.wvx * s;
-      for (int i = 0; i < n; ++i) lxx[i * n + i] = clip0(eps);
-      lx[2] = z2 * (x[2] - P.znom); lxx[2 * n + 2] = z2 > eps ? z2 : eps;
-      for (int k = 3; k < 6; ++k) { lx[k] = r2 * x[k]; lxx[k * n + k] = r2 > eps ? r2 : eps; }
-      lx[N] = x2 * (x[N] - P.vxt); lxx[N * n + N] = x2 > eps ? x2 : eps;
+      for (int i = g.lane; i < n; i += G) {
+        const R d = i == 2 ? z2 : i >= 3 && i < 6 ? r2 : i == N ? x2 : R(0);
+        lxx[i * n + i] = i == 2 || (i >= 3 && i < 6) || i == N ? (d > eps ? d : eps) : clip0(eps);
+        if (i == 2) lx[i] = z2 * (x[2] - P.znom);
+        else if (i >= 3 && i < 6) lx[i] = r2 * x[i];
+        else if (i == N) lx[i] = x2 * (x[N] - P.vxt);
+      }
     }
   }
 
