@@ -995,7 +995,6 @@ struct Solver {
   TO_DEV static int backward_knot(const Params& P, const Group<G>& g, W& w, bool act, bool act_next,
                                   const SolveArgs& a, R (&pb)[PB], const R* trec_next, R* grec, double* vxrec,
                                   double mu_lm, bool timer, long long& tlast, const R* kprim, const BlockDst& dst, const Spread& sp) {
-    const R eps = (R)a.eps;
     if constexpr (!Sys::kStoredDerivs && !Sys::kGainDerivs) {   // x_k, u_k feed the derivative step (stored blocks need neither)
       if (act) {
 #pragma unroll
@@ -1055,7 +1054,7 @@ struct Solver {
         if (act_next && e < Sys::kBlock) pb[s] = kprim[e];
       }
     } else if (act) {
-      Sys::template derivs_staged<R, G>(P, g, w.xk, w.uk, eps, w.A, w.Bm, w.lxx, w.lx, w.luu, w.lu, w.sx, kprim);
+      Sys::template derivs_staged<R, G>(P, g, w.xk, w.uk, w.A, w.Bm, w.lx, w.lu, w.sx, kprim);
     }
     g.sync();
     TO_TICK(1);
@@ -1670,6 +1669,8 @@ struct Solver {
             g.sync();
             if (bw && a.vx && a.want_vx)
               for (int i = g.lane; i < n; i += G) vx_at(a, a.vx, base + T)[i] = (double)w.v[i];
+            // (one lane used to rewrite the constant Hessians at every knot)
+            if (bw) Sys::running_consts(P, g.lane, G, (R)a.eps, w.lxx, w.lx, w.luu);
             // every lane: the substep primal chains of its knots (bw is uniform over a group of whole warps)
             if (bw)
               for (int k = g.lane; k < T; k += G) {

@@ -744,28 +744,38 @@ struct SysRigid {
     return l;
   }
 
-  // separable running costs: the clipped Hessians are diagonal, max(d, eps)
+  // Separable running costs: the clipped Hessians are diagonal, max(d, eps), and
+  // the same at every knot, so they are set once a pass; a knot's gradients are
+  // linear in x and u.  By the lanes of the group.
   template <class R>
-  TO_DEV static void running_derivs(const ParamsT<R>& P, const R* x, const R* u, R eps, R* lxx, R* lx, R* luu,
-                                    R* lu) {
-    for (int i = 0; i < n * n; ++i) lxx[i] = 0;
-    for (int i = 0; i < m * m; ++i) luu[i] = 0;
-    for (int i = 0; i < n; ++i) lx[i] = 0;
+  TO_DEV static void running_consts(const ParamsT<R>& P, int lane, int G, R eps, R* lxx, R* lx, R* luu) {
     const R w2 = R(2) * P.wtau;
-    for (int j = 0; j < m; ++j) { lu[j] = w2 * u[j]; luu[j * m + j] = w2 > eps ? w2 : eps; }
-    R dq[N];   // diagonal of the q-block and qd-block
-    for (int i = 0; i < n; ++i) lxx[i * n + i] = clip0(eps);
-    if (KIND == RK_ARM7) {
-      const R v2 = R(2) * P.wv;
-#pragma unroll
-      for (int j = 0; j < N; ++j) { lx[N + j] = v2 * x[N + j]; lxx[(N + j) * n + N + j] = v2 > eps ? v2 : eps; }
-    } else {
-      const R z2 = R(2) * P.wz, r2 = R(2) * P.wrpy, x2 = R(2) * P.wvx;
-      lx[2] = z2 * (x[2] - P.znom); lxx[2 * n + 2] = z2 > eps ? z2 : eps;
-      for (int k = 3; k < 6; ++k) { lx[k] = r2 * x[k]; lxx[k * n + k] = r2 > eps ? r2 : eps; }
-      lx[N] = x2 * (x[N] - P.vxt); lxx[N * n + N] = x2 > eps ? x2 : eps;
+    for (int e = lane; e < n * n; e += G) {
+      const int i = e / n;
+      R d = R(0);
+      bool cost = false;
+      if (KIND == RK_ARM7) {
+        cost = i >= N;
+        d = R(2) * P.wv;
+      } else {
+        cost = i == 2 || (i >= 3 && i < 6) || i == N;
+        d = R(2) * (i == 2 ? P.wz : i == N ? P.wvx : P.wrpy);
+      }
+      lxx[e] = i != e % n ? R(0) : cost ? (d > eps ? d : eps) : clip0(eps);
     }
-    (void)dq;
+    for (int e = lane; e < m * m; e += G) luu[e] = e / m != e % m ? R(0) : (w2 > eps ? w2 : eps);
+    for (int e = lane; e < n; e += G) lx[e] = R(0);
+  }
+  template <class R, int G>
+  TO_DEV static void running_grads(const ParamsT<R>& P, int lane, const R* x, const R* u, R* lx, R* lu) {
+    for (int i = lane; i < m; i += G) lu[i] = (R(2) * P.wtau) * u[i];
+    if (KIND == RK_ARM7) {
+      for (int i = lane; i < N; i += G) lx[N + i] = (R(2) * P.wv) * x[N + i];
+    } else {
+      if (lane == 2) lx[2] = (R(2) * P.wz) * (x[2] - P.znom);
+      else if (lane >= 3 && lane < 6) lx[lane] = (R(2) * P.wrpy) * x[lane];
+      else if (lane == 6) lx[N] = (R(2) * P.wvx) * (x[N] - P.vxt);
+    }
   }
 
   // Terminal-cost derivatives (V and v in shared memory), by a group of whole
@@ -1274,8 +1284,8 @@ struct SysRigid {
   // narrower than the n + m directions takes them in passes of G (the
   // substeps are staged again for each pass).
   template <class R, int G>
-  TO_DEV static void derivs_staged(const ParamsT<R>& P, const Group<G>& g, const R* x, const R* u, R eps, R* A, R* B,
-                                   R* lxx, R* lx, R* luu, R* lu, R* scratch, const R* prims) {
+  TO_DEV static void derivs_staged(const ParamsT<R>& P, const Group<G>& g, const R* x, const R* u, R* A, R* B, R* lx,
+                                   R* lu, R* scratch, const R* prims) {
     for (int pass = 0; pass < (n + m + G - 1) / G; ++pass) {
     if (pass > 0) g.sync();   // every lane done with the staging buffers of the previous pass
     const int c = pass * G + g.lane;
@@ -1318,7 +1328,7 @@ struct SysRigid {
       }
     }
     }
-    if (g.lane == G - 1) running_derivs(P, x, u, eps, lxx, lx, luu, lu);
+    running_grads<R, G>(P, g.lane, x, u, lx, lu);
   }
 
 };
