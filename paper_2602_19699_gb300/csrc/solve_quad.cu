@@ -26,6 +26,13 @@ static int parse_quad(const double* p, size_t np, std::vector<unsigned char>& bl
     if (P.foot_body[f] != RigidTopo<RK_QUAD>::foot_body(f)) { err = "quad params: foot f must be on calf body 8 + 3 f"; return -1; }
     for (int k = 0; k < 3; ++k) P.foot_pt[f][k] = c[12 + 4 * f + k];
   }
+  // joints 0..5 only place the base: no mass before body 5, every joint at one point
+  P.free_base = 1;
+  for (int i = 0; i < 6; ++i)
+    for (int k = 0; k < 3; ++k) {
+      if (P.off[i][k] != 0) P.free_base = 0;
+      if (i < 5 && (P.mass[i] != 0 || P.inertia[i][k] != 0)) P.free_base = 0;
+    }
   to_blobs<RigidQuadP>(P, blob64, blob32);
   return 0;
 }
