@@ -1455,155 +1455,214 @@ struct SysRigid {
   // recursion (velocities, accelerations, body forces, world poses and
   // contact) and the backward force recursion.  Only the tangents live in
   // the lane's own arrays.
+  // One body of the forward recursion: its tangents and its force's from its
+  // parent's (pa < 0: none).
+  template <class R>
+  TO_DEV static void tan_body(const ParamsT<R>& P, const Prim<R>& pr, int jt, int i, int pa, R dq, R dqd, const R* pdvw,
+                              const R* pdvv, const R* pdaw, const R* pdav, R* dvw, R* dvv, R* daw, R* dav, R* dfn, R* dff) {
+    const bool rev = jt <= 2;
+    const int ax = rev ? jt : jt - 3;
+    const R* E = pr.E[i];
+    const R* r = pr.r[i];
+    R t[3];
+    if (pa < 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) { dvw[k] = R(0); dvv[k] = R(0); daw[k] = R(0); dav[k] = R(0); }
+    } else {
+      R pw[3], paw[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) { pw[k] = pr.vw[pa][k]; paw[k] = pr.aw[pa][k]; }
+      // velocity
+      jmv(jt, E, pdvw, dvw);
+      if (rev) rot_tangent(ax, dq, pr.Epw[i], dvw);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) t[k] = pdvv[k];
+      cross_sub(r, pdvw, t);
+      if (!rev) axis_acc(pw, ax, dq, t);
+      jmv(jt, E, t, dvv);
+      if (rev) rot_tangent(ax, dq, pr.Ept[i], dvv);
+      // acceleration (qdd fixed)
+      jmv(jt, E, pdaw, daw);
+      if (rev) rot_tangent(ax, dq, pr.Epa[i], daw);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) t[k] = pdav[k];
+      cross_sub(r, pdaw, t);
+      if (!rev) axis_acc(paw, ax, dq, t);
+      jmv(jt, E, t, dav);
+    }
+    if (rev) rot_tangent(ax, dq, pr.Epb[i], dav);
+    if (rev) dvw[ax] += dqd; else dvv[ax] += dqd;
+    if (pa >= 0) {
+      if (rev) {
+        axis_acc(dvw, ax, pr.qd[i], daw);
+        axis_acc(pr.vw[i], ax, dqd, daw);
+        axis_acc(dvv, ax, pr.qd[i], dav);
+        axis_acc(pr.vv[i], ax, dqd, dav);
+      } else {
+        axis_acc(dvw, ax, pr.qd[i], dav);
+        axis_acc(pr.vw[i], ax, dqd, dav);
+      }
+    }
+    // body force
+    R dhn[3], dhf[3];
+    inertia_mul(P, i, daw, dav, dfn, dff);
+    inertia_mul(P, i, dvw, dvv, dhn, dhf);
+    cross_acc(dvw, pr.hn[i], dfn);
+    cross_acc(pr.vw[i], dhn, dfn);
+    cross_acc(dvv, pr.hf[i], dfn);
+    cross_acc(pr.vv[i], dhf, dfn);
+    cross_acc(dvw, pr.hf[i], dff);
+    cross_acc(pr.vw[i], dhf, dff);
+  }
+  // its world pose's: dE0_i = dE_i E0_p + E_i dE0_p, dp0_i = dp0_p + dE0_p^T r + E0_p^T dr
+  template <class R>
+  TO_DEV static void tan_pose(const Prim<R>& pr, int jt, int i, int pa, R dq, const R* pdE0, const R* pdp0, R* dE0, R* dp0) {
+    const bool rev = jt <= 2;
+    const int ax = rev ? jt : jt - 3;
+    if (pa < 0) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) dE0[k] = R(0);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) dp0[k] = !rev && k == ax ? dq : R(0);
+    } else {
+      const R* E = pr.E[i];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) dE0[a * 3 + b] = e_row(jt, E, pdE0, a, b);
+      R w1[3];
+      mtv(pdE0, pr.r[i], w1);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) dp0[k] = pdp0[k] + w1[k];
+      if (!rev)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) dp0[k] += pr.E0[pa][ax * 3 + k] * dq;
+    }
+    if (rev) {
+      // column b of E0_i turns with the joint: -dq (e_ax x column)
+      const R* E0 = pr.E0[i];
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const R col[3] = {E0[0 * 3 + b], E0[1 * 3 + b], E0[2 * 3 + b]};
+        R y[3] = {dE0[0 * 3 + b], dE0[1 * 3 + b], dE0[2 * 3 + b]};
+        rot_tangent(ax, dq, col, y);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) dE0[a * 3 + b] = y[a];
+      }
+    }
+  }
+  // the contact force of foot ft on body bi
+  template <class R>
+  TO_DEV static void tan_contact(const ParamsT<R>& P, const Prim<R>& pr, int ft, int bi, const R* dE0, const R* dp0,
+                                 const R* dvw, const R* dvv, R* dfn, R* dff) {
+    const R pt[3] = {P.foot_pt[ft][0], P.foot_pt[ft][1], P.foot_pt[ft][2]};
+    const R* E0 = pr.E0[bi];
+    R dwpt[3], dvb[3], dvwld[3], w1[3];
+    mtv(dE0, pt, dwpt);
+    const R dz = dp0[2] + dwpt[2];
+    cross(dvw, pt, w1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dvb[k] = dvv[k] + w1[k];
+    mtv(dE0, pr.vb[ft], dvwld);
+    mtv(E0, dvb, w1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dvwld[k] += w1[k];
+    const R gate = pr.gate[ft];
+    const R dgate = -P.beta * gate * (R(1) - gate) * dz;
+    const R dsp = -gate * dz;
+    R dF[3];
+    dF[0] = -P.dc * (dgate * pr.vwld[ft][0] + gate * dvwld[0]);
+    dF[1] = -P.dc * (dgate * pr.vwld[ft][1] + gate * dvwld[1]);
+    dF[2] = P.kc * dsp - P.dc * (dgate * pr.vwld[ft][2] + gate * dvwld[2]);
+    R mw[3], dmw[3] = {R(0), R(0), R(0)}, dmb[3], dfb[3];
+    cross(pr.wpt[ft], pr.F[ft], mw);
+    cross_acc(dwpt, pr.F[ft], dmw);
+    cross_acc(pr.wpt[ft], dF, dmw);
+    mv(dE0, mw, dmb);
+    mv(E0, dmw, w1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dmb[k] += w1[k];
+    mv(dE0, pr.F[ft], dfb);
+    mv(E0, dF, w1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { dfn[k] -= dmb[k]; dff[k] -= dfb[k] + w1[k]; }
+  }
+  // a body's force tangent added to its parent's:
+  // d(E^T y) = E^T dy + dq E^T (e_ax x y) for a revolute joint
+  template <class R>
+  TO_DEV static void tan_up(const Prim<R>& pr, int jt, int i, R dq, const R* dfn, const R* dff, R* pfn, R* pff) {
+    const bool rev = jt <= 2;
+    const int ax = rev ? jt : jt - 3;
+    const R* E = pr.E[i];
+    R yn[3], yf[3], den[3], def[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { yn[k] = dfn[k]; yf[k] = dff[k]; }
+    if (rev) {
+      rot_tangent(ax, -dq, pr.fn[i], yn);
+      rot_tangent(ax, -dq, pr.ff[i], yf);
+    }
+    jmtv(jt, E, yn, den);
+    jmtv(jt, E, yf, def);
+    if (!rev) {
+      R ef[3];
+      jmtv(jt, E, pr.ff[i], ef);
+      axis_acc(ef, ax, -dq, den);
+    }
+    cross_acc(pr.r[i], def, den);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { pfn[k] += den[k]; pff[k] += def[k]; }
+  }
+
   template <class R>
   TO_DEV static void rnea_tangent(const ParamsT<R>& P, const Prim<R>& pr, const R* dq, const R* dqd, R* dtau) {
-    R dvw[N][3], dvv[N][3], daw[N][3], dav[N][3], dfn[N][3], dff[N][3];
-    R dE0[KIND == RK_QUAD ? N : 1][9], dp0[KIND == RK_QUAD ? N : 1][3];
+    constexpr int NB = KIND == RK_QUAD ? 6 : N;     // bodies of the chain that the pass unrolls
+    R dvw[NB][3], dvv[NB][3], daw[NB][3], dav[NB][3], dfn[NB][3], dff[NB][3];
+    R dE0[KIND == RK_QUAD ? NB : 1][9], dp0[KIND == RK_QUAD ? NB : 1][3];
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const int pa = parent(i);
-      const int jt = jtype(i);
-      const bool rev = jt <= 2;
-      const int ax = rev ? jt : jt - 3;
-      R dr[3] = {R(0), R(0), R(0)};
-      if (!rev) dr[ax] = dq[i];
-      const R* E = pr.E[i];
-      const R* r = pr.r[i];
-      R t[3];
-      if (pa < 0) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) { dvw[i][k] = R(0); dvv[i][k] = R(0); daw[i][k] = R(0); dav[i][k] = R(0); }
-      } else {
-        R pw[3], paw[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) { pw[k] = pr.vw[pa][k]; paw[k] = pr.aw[pa][k]; }
-        // velocity
-        jmv(jt, E, dvw[pa], dvw[i]);
-        if (rev) rot_tangent(ax, dq[i], pr.Epw[i], dvw[i]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) t[k] = dvv[pa][k];
-        cross_sub(r, dvw[pa], t);
-        if (!rev) axis_acc(pw, ax, dq[i], t);
-        jmv(jt, E, t, dvv[i]);
-        if (rev) rot_tangent(ax, dq[i], pr.Ept[i], dvv[i]);
-        // acceleration (qdd fixed)
-        jmv(jt, E, daw[pa], daw[i]);
-        if (rev) rot_tangent(ax, dq[i], pr.Epa[i], daw[i]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) t[k] = dav[pa][k];
-        cross_sub(r, daw[pa], t);
-        if (!rev) axis_acc(paw, ax, dq[i], t);
-        jmv(jt, E, t, dav[i]);
-      }
-      if (rev) rot_tangent(ax, dq[i], pr.Epb[i], dav[i]);
-      if (rev) dvw[i][ax] += dqd[i]; else dvv[i][ax] += dqd[i];
-      if (pa >= 0) {
-        if (rev) {
-          axis_acc(dvw[i], ax, pr.qd[i], daw[i]);
-          axis_acc(pr.vw[i], ax, dqd[i], daw[i]);
-          axis_acc(dvv[i], ax, pr.qd[i], dav[i]);
-          axis_acc(pr.vv[i], ax, dqd[i], dav[i]);
-        } else {
-          axis_acc(dvw[i], ax, pr.qd[i], dav[i]);
-          axis_acc(pr.vw[i], ax, dqd[i], dav[i]);
-        }
-      }
-      // body force
-      R dIn[3], dIf[3], dhn[3], dhf[3];
-      inertia_mul(P, i, daw[i], dav[i], dIn, dIf);
-      inertia_mul(P, i, dvw[i], dvv[i], dhn, dhf);
-      for (int k = 0; k < 3; ++k) { dfn[i][k] = dIn[k]; dff[i][k] = dIf[k]; }
-      cross_acc(dvw[i], pr.hn[i], dfn[i]);
-      cross_acc(pr.vw[i], dhn, dfn[i]);
-      cross_acc(dvv[i], pr.hf[i], dfn[i]);
-      cross_acc(pr.vv[i], dhf, dfn[i]);
-      cross_acc(dvw[i], pr.hf[i], dff[i]);
-      cross_acc(pr.vw[i], dhf, dff[i]);
-      if (KIND == RK_QUAD) {
-        // world pose: dE0_i = dE_i E0_p + E_i dE0_p, dp0_i = dp0_p + dE0_p^T r + E0_p^T dr
-        const R* E0 = pr.E0[i];
-        if (pa < 0) {
-          for (int k = 0; k < 9; ++k) dE0[i][k] = R(0);
-          for (int k = 0; k < 3; ++k) dp0[i][k] = dr[k];
-        } else {
-          for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) dE0[i][a * 3 + b] = e_row(jt, E, dE0[pa], a, b);
-          R w1[3], w2[3];
-          mtv(dE0[pa], r, w1);
-          mtv(pr.E0[pa], dr, w2);
-          for (int k = 0; k < 3; ++k) dp0[i][k] = dp0[pa][k] + w1[k] + w2[k];
-        }
-        if (rev) {
-          // column b of E0_i turns with the joint: -dq (e_ax x column)
-          for (int b = 0; b < 3; ++b) {
-            const R col[3] = {E0[0 * 3 + b], E0[1 * 3 + b], E0[2 * 3 + b]};
-            R y[3] = {R(0), R(0), R(0)};
-            rot_tangent(ax, dq[i], col, y);
-            for (int a = 0; a < 3; ++a) dE0[i][a * 3 + b] += y[a];
-          }
-        }
-      }
+    for (int i = 0; i < NB; ++i) {
+      const int pa = parent(i), pb = pa < 0 ? 0 : pa;
+      tan_body(P, pr, jtype(i), i, pa, dq[i], dqd[i], dvw[pb], dvv[pb], daw[pb], dav[pb], dvw[i], dvv[i], daw[i], dav[i],
+               dfn[i], dff[i]);
+      if constexpr (KIND == RK_QUAD) tan_pose(pr, jtype(i), i, pa, dq[i], dE0[pb], dp0[pb], dE0[i], dp0[i]);
     }
-    if (KIND == RK_QUAD) {
+    if constexpr (KIND == RK_QUAD) {
+      // The legs one after another in a loop: the body index is data, so their
+      // code is there once, and only one leg's tangents are live.  Unrolled, the
+      // 18 bodies' arrays did not fit the registers and the warps waited for
+      // their spills and for instructions: B=512 float32, T 4..8, 1 iteration, V_x
+      // 7.8 -> 6.8 ms.
+#pragma unroll 1
+      for (int leg = 3; leg >= 0; --leg) {
+        const int b = 6 + 3 * leg;
+        auto pick = [&](const R* d, int k) { return leg == 0 ? d[6 + k] : leg == 1 ? d[9 + k] : leg == 2 ? d[12 + k] : d[15 + k]; };
+        R lw[3][3], lv[3][3], la[3][3], lb[3][3], ln[3][3], lf[3][3], lE[9], lp[3], mE[9], mp[3], lq[3], lqd[3];
 #pragma unroll
-      for (int ft = 0; ft < kFeet; ++ft) {
-        const int bi = foot_body(ft);
-        const R pt[3] = {P.foot_pt[ft][0], P.foot_pt[ft][1], P.foot_pt[ft][2]};
-        const R* E0 = pr.E0[bi];
-        R dwpt[3], dvb[3], dvwld[3], w1[3];
-        mtv(dE0[bi], pt, dwpt);
-        const R dz = dp0[bi][2] + dwpt[2];
-        cross(dvw[bi], pt, w1);
-        for (int k = 0; k < 3; ++k) dvb[k] = dvv[bi][k] + w1[k];
-        mtv(dE0[bi], pr.vb[ft], dvwld);
-        mtv(E0, dvb, w1);
-        for (int k = 0; k < 3; ++k) dvwld[k] += w1[k];
-        const R gate = pr.gate[ft];
-        const R dgate = -P.beta * gate * (R(1) - gate) * dz;
-        const R dsp = -gate * dz;
-        R dF[3];
-        dF[0] = -P.dc * (dgate * pr.vwld[ft][0] + gate * dvwld[0]);
-        dF[1] = -P.dc * (dgate * pr.vwld[ft][1] + gate * dvwld[1]);
-        dF[2] = P.kc * dsp - P.dc * (dgate * pr.vwld[ft][2] + gate * dvwld[2]);
-        R mw[3], dmw[3] = {R(0), R(0), R(0)}, dmb[3], dfb[3];
-        cross(pr.wpt[ft], pr.F[ft], mw);
-        cross_acc(dwpt, pr.F[ft], dmw);
-        cross_acc(pr.wpt[ft], dF, dmw);
-        mv(dE0[bi], mw, dmb);
-        mv(E0, dmw, w1);
-        for (int k = 0; k < 3; ++k) dmb[k] += w1[k];
-        mv(dE0[bi], pr.F[ft], dfb);
-        mv(E0, dF, w1);
-        for (int k = 0; k < 3; ++k) dfb[k] += w1[k];
-        for (int k = 0; k < 3; ++k) { dfn[bi][k] -= dmb[k]; dff[bi][k] -= dfb[k]; }
+        for (int k = 0; k < 3; ++k) { lq[k] = pick(dq, k); lqd[k] = pick(dqd, k); }
+        tan_body(P, pr, 0, b, 5, lq[0], lqd[0], dvw[5], dvv[5], daw[5], dav[5], lw[0], lv[0], la[0], lb[0], ln[0], lf[0]);
+        tan_pose(pr, 0, b, 5, lq[0], dE0[5], dp0[5], lE, lp);
+        tan_body(P, pr, 1, b + 1, b, lq[1], lqd[1], lw[0], lv[0], la[0], lb[0], lw[1], lv[1], la[1], lb[1], ln[1], lf[1]);
+        tan_pose(pr, 1, b + 1, b, lq[1], lE, lp, mE, mp);
+        tan_body(P, pr, 1, b + 2, b + 1, lq[2], lqd[2], lw[1], lv[1], la[1], lb[1], lw[2], lv[2], la[2], lb[2], ln[2], lf[2]);
+        tan_pose(pr, 1, b + 2, b + 1, lq[2], mE, mp, lE, lp);
+        tan_contact(P, pr, leg, b + 2, lE, lp, lw[2], lv[2], ln[2], lf[2]);
+        R t[3];
+        t[2] = ln[2][1];
+        tan_up(pr, 1, b + 2, lq[2], ln[2], lf[2], ln[1], lf[1]);
+        t[1] = ln[1][1];
+        tan_up(pr, 1, b + 1, lq[1], ln[1], lf[1], ln[0], lf[0]);
+        t[0] = ln[0][0];
+        tan_up(pr, 0, b, lq[0], ln[0], lf[0], dfn[5], dff[5]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) dtau[6 + 3 * j + k] = j == leg ? t[k] : dtau[6 + 3 * j + k];
       }
     }
 #pragma unroll
-    for (int i = N - 1; i >= 0; --i) {
-      const int jt = jtype(i);
-      const bool rev = jt <= 2;
-      const int ax = rev ? jt : jt - 3;
-      dtau[i] = rev ? dfn[i][ax] : dff[i][ax];
-      const int pa = parent(i);
-      if (pa >= 0) {
-        // d(E^T y) = E^T dy + dq E^T (e_ax x y) for a revolute joint
-        const R* E = pr.E[i];
-        R yn[3], yf[3], den[3], def[3];
-        for (int k = 0; k < 3; ++k) { yn[k] = dfn[i][k]; yf[k] = dff[i][k]; }
-        if (rev) {
-          rot_tangent(ax, -dq[i], pr.fn[i], yn);
-          rot_tangent(ax, -dq[i], pr.ff[i], yf);
-        }
-        jmtv(jt, E, yn, den);
-        jmtv(jt, E, yf, def);
-        if (!rev) {
-          R ef[3];
-          jmtv(jt, E, pr.ff[i], ef);
-          axis_acc(ef, ax, -dq[i], den);
-        }
-        cross_acc(pr.r[i], def, den);
-        for (int k = 0; k < 3; ++k) { dfn[pa][k] += den[k]; dff[pa][k] += def[k]; }
-      }
+    for (int i = NB - 1; i >= 0; --i) {
+      const int jt = jtype(i), pa = parent(i);
+      dtau[i] = jt <= 2 ? dfn[i][jt <= 2 ? jt : 0] : dff[i][jt <= 2 ? 0 : jt - 3];
+      if (pa >= 0) tan_up(pr, jt, i, dq[i], dfn[i], dff[i], dfn[pa], dff[pa]);
     }
   }
 
