@@ -159,6 +159,13 @@ struct SysRigid {
   static constexpr int anc(int i, int d) { return Topo::anc(i, d); }
   static constexpr int foot_body(int f) { return Topo::foot_body(f); }
 
+  // a body without mass needs no force of its own (the joints that place the
+  // quadruped's base: 5 of 18 bodies; uniform over the grid)
+  template <class R> TO_DEV static bool massless(const ParamsT<R>& P, int i) {
+    if constexpr (KIND == RK_QUAD) return P.free_base && i < 5;
+    else return false;
+  }
+
   // 3-vectors
   template <class S> TO_DEV static void cross(const S* a, const S* b, S* c) {
     const S c0 = a[1] * b[2] - a[2] * b[1], c1 = a[2] * b[0] - a[0] * b[2], c2 = a[0] * b[1] - a[1] * b[0];
@@ -374,6 +381,11 @@ struct SysRigid {
       } else {
         axis_acc(vw, ax, qd, av);
       }
+    }
+    if (massless(P, i)) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) { hn[k] = R(0); hf[k] = R(0); fn[k] = R(0); ff[k] = R(0); }
+      return;
     }
     inertia_mul(P, i, aw, av, fn, ff);
     inertia_mul(P, i, vw, vv, hn, hf);
@@ -1412,6 +1424,11 @@ struct SysRigid {
       if (jt <= 2) aw[jt] += pr.qdd[i]; else av[i][jt - 3] += pr.qdd[i];
 #pragma unroll
       for (int k = 0; k < 3; ++k) pr.aw[i][k] = aw[k];
+      if (massless(P, i)) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { fn[i][k] = R(0); ff[i][k] = R(0); }
+        continue;
+      }
       R In[3], If[3];
       inertia_mul(P, i, aw, av[i], In, If);
 #pragma unroll
@@ -1504,6 +1521,11 @@ struct SysRigid {
       }
     }
     // body force
+    if (massless(P, i)) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) { dfn[k] = R(0); dff[k] = R(0); }
+      return;
+    }
     R dhn[3], dhf[3];
     inertia_mul(P, i, daw, dav, dfn, dff);
     inertia_mul(P, i, dvw, dvv, dhn, dhf);
