@@ -99,7 +99,8 @@ TO_DEV void semi_implicit2(R* qh, R* ql, R* vh, R* vl, const R* a, R h) {
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     acc2(vh[i], vl[i], h * a[i]);
-    acc2(qh[i], ql[i], h * vh[i] + h * vl[i]);
+    if constexpr (sizeof(R) == 4) acc2(qh[i], ql[i], h * vh[i] + h * vl[i]);
+    else qh[i] += h * vh[i];             // (float64 states have no low part)
   }
 }
 

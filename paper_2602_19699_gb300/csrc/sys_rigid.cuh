@@ -159,6 +159,10 @@ struct SysRigid {
   static constexpr int anc(int i, int d) { return Topo::anc(i, d); }
   static constexpr int foot_body(int f) { return Topo::foot_body(f); }
 
+  // the arm's float32 solves are chaotic: code that would round otherwise than
+  // the rest of a solve was rounded before is not used there
+  template <class R> static constexpr bool kKeepBits = KIND == RK_ARM7 && sizeof(R) == 4;
+
   // a body without mass needs no force of its own (the joints that place the
   // quadruped's base: 5 of 18 bodies; uniform over the grid)
   template <class R> TO_DEV static bool massless(const ParamsT<R>& P, int i) {
@@ -394,11 +398,12 @@ struct SysRigid {
     cross_acc(vw, hf, ff);
   }
 
-  // the bias torques: inverse dynamics at qdd = 0 with gravity and contact
+  // the bias torques: inverse dynamics at qdd = 0 with gravity and contact; the
+  // joint transforms are left in E and r
   template <class R, class S>
-  TO_DEV static void rnea(const ParamsT<R>& P, const S* q, const S* qd, S* tau) {
+  TO_DEV static void rnea(const ParamsT<R>& P, const S* q, const S* qd, S* tau, S (*E)[9], S (*r)[3]) {
     constexpr bool contact = KIND == RK_QUAD;
-    S E[N][9], r[N][3], vw[N][3], vv[N][3], fn[N][3], ff[N][3];
+    S vw[N][3], vv[N][3], fn[N][3], ff[N][3];
     S E0[KIND == RK_QUAD ? N : 1][9], p0[KIND == RK_QUAD ? N : 1][3];
     S awb[N][3], avb[N][3];
 #pragma unroll
@@ -490,15 +495,28 @@ struct SysRigid {
   // as (mass, first moment h = mass * com, rotational inertia about the
   // origin); moving it to the parent frame rotates it and applies the
   // parallel-axis shift.  Bodies are ordered parents first.
+  // Eb, rb (nullable): the joint transforms of q from its bias pass.  A step
+  // evaluated each sine and cosine twice, 25 FP64 instructions a joint (float64
+  // arm, B = 304, T = 10 to 20: 8.93 -> 8.54 ms with the fused position update;
+  // quadruped, B = 512, T = 4 to 8: 6.79 -> 6.60 ms).  The
+  // float32 arm still does: with shared transforms the compiler fuses other
+  // multiply-adds, and the results are no longer the same bits.
   template <class R>
-  TO_DEV static void mass_chol(const ParamsT<R>& P, const R* q, R* L) {
-    // the arm's float32 solves are chaotic and keep the full products' bits
-    constexpr bool kFull = KIND == RK_ARM7 && sizeof(R) == 4;
+  TO_DEV static void mass_chol(const ParamsT<R>& P, const R* q, R* L, const R (*Eb)[9] = nullptr,
+                               const R (*rb)[3] = nullptr) {
+    constexpr bool kFull = kKeepBits<R>;   // the full products of a joint transform
     R E[N][9], r[N][3];
     R cm[N], ch[N][3], cI[N][6];   // cI: xx, yy, zz, xy, xz, yz
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      joint_transform(P, i, q[i], E[i], r[i]);
+      if (!Eb) {
+        joint_transform(P, i, q[i], E[i], r[i]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) E[i][k] = Eb[i][k];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) r[i][k] = rb[i][k];
+      }
       const R mi = P.mass[i], c0 = P.com[i][0], c1 = P.com[i][1], c2 = P.com[i][2];
       cm[i] = mi;
       ch[i][0] = mi * c0; ch[i][1] = mi * c1; ch[i][2] = mi * c2;
@@ -649,9 +667,10 @@ struct SysRigid {
   // one substep's acceleration: qdd = M^{-1} (tau - h); also returns L
   template <class R>
   TO_DEV static void accel(const ParamsT<R>& P, const R* q, const R* qd, const R* tau, R* qdd, R* L) {
-    R h[N], rhs[N];
-    rnea<R, R>(P, q, qd, h);
-    mass_chol(P, q, L);
+    R h[N], rhs[N], E[N][9], r[N][3];
+    rnea<R, R>(P, q, qd, h, E, r);
+    if constexpr (kKeepBits<R>) mass_chol(P, q, L);
+    else mass_chol(P, q, L, E, r);
 #pragma unroll
     for (int i = 0; i < N; ++i) rhs[i] = tau[i] - h[i];
     chol_solve(P, L, rhs, qdd);
@@ -1098,7 +1117,8 @@ struct SysRigid {
       g.sync();
       R hb[N];
       if (mine) {
-        rnea<R, R>(P, xh, xh + N, hb);
+        R E[N][9], r[N][3];
+        rnea<R, R>(P, xh, xh + N, hb, E, r);
       } else if (c >= H && slot < kStepSlots && flag[slot] != R(0)) {
         mass_chol_mem(P, sq, sL);
       }
@@ -1290,13 +1310,16 @@ struct SysRigid {
   // reads them all from pr):
   // bias_store (one lane): those quantities, I v, and the inverse dynamics at
   // qdd = 0 (gravity, velocity products, contact), i.e. the bias torques h.
+  // The joint transforms are also left in Ej and rj.
   template <class R>
-  TO_DEV static void bias_store(const ParamsT<R>& P, Prim<R>& pr, const R* q, const R* qd, R* h) {
+  TO_DEV static void bias_store(const ParamsT<R>& P, Prim<R>& pr, const R* q, const R* qd, R* h, R (*Ej)[9],
+                                R (*rj)[3]) {
     R aw[N][3], av[N][3], fn[N][3], ff[N][3];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int pa = parent(i), jt = jtype(i);
-      R E[9], r[3];
+      R* E = Ej[i];
+      R* r = rj[i];
       joint_transform(P, i, q[i], E, r);
 #pragma unroll
       for (int k = 0; k < 9; ++k) pr.E[i][k] = E[k];
@@ -1699,9 +1722,10 @@ struct SysRigid {
     const R h = P.dt / (R)P.n_sub;
     for (int s = 0; s < P.n_sub; ++s) {
       Prim<R>& pr = *reinterpret_cast<Prim<R>*>(out + (size_t)s * kPrimStride<R>);
-      R hb[N], L[N * N], rhs[N], qdd[N];
-      bias_store(P, pr, q, qd, hb);
-      mass_chol(P, q, L);
+      R hb[N], L[N * N], rhs[N], qdd[N], E[N][9], r[N][3];
+      bias_store(P, pr, q, qd, hb, E, r);
+      if constexpr (kKeepBits<R>) mass_chol(P, q, L);
+      else mass_chol(P, q, L, E, r);
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         pr.L[k * N + k] = L[k * N + k];
