@@ -461,8 +461,9 @@ int totune(to_problem p, int B, const double* x0, const int* T, to_solver_opts* 
  * solve of n member batches (one per problem, member i solving B[i]
  * instances): per member, the host-to-device copies of x0 and T from pinned
  * staging that the graph owns, the horizon sort, the persistent solver
- * kernel, the gather of X and U (when want_traj) and the device-to-host
- * copies of X, U, J, iters and status into pinned staging.  The members'
+ * kernel, X and U straight into pinned staging (when want_traj: by the
+ * solver as each instance is done, or by the gather that follows it) and the
+ * device-to-host copies of J, iters and status.  The members'
  * branches are independent, so their kernels run at the same time, each
  * sized to its share of the resident CTAs (shares[i] / sum(shares); shares
  * NULL = equal).  Horizons may change between launches (the sort runs on the

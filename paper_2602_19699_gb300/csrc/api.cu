@@ -119,43 +119,66 @@ __global__ void prepare_kernel(int B, const int* __restrict__ T, int T_max, long
 // [1, T_max] or more knots than the workspace) ran no solve, so its offsets
 // and slots are not valid: every output is NaN and nothing is read.  The
 // horizon and slot are clamped to their ranges before use either way.
+//
+// Bound by memory.  A block takes an instance (grid.y) and a stretch of its
+// output elements, one thread each, so that every store and, within a record,
+// every load is of consecutive addresses (one thread per knot, as before,
+// stored 8 bytes every 48).  rows_done: the solver has written the rows up to
+// the horizon (SolveArgs.X_out, U_out), the padding remains.
 __global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, int NS, int rbytes,
                               const long long* __restrict__ toff, const int* __restrict__ T,
                               const int* __restrict__ slot,
                               const void* __restrict__ traj, const void* __restrict__ gains,
                               const double* __restrict__ vx, double* __restrict__ X, double* __restrict__ U,
-                              double* __restrict__ Vx, double* __restrict__ K, const int* __restrict__ err) {
-  const long long total = (long long)B * (T_max + 1);
+                              double* __restrict__ Vx, double* __restrict__ K, const int* __restrict__ err,
+                              bool rows_done) {
   const bool rejected = err && *err;
   const double qnan = __longlong_as_double(0x7ff8000000000000LL);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(t / (T_max + 1));
-    const int k = (int)(t % (T_max + 1));
+  const int e0 = blockIdx.x * blockDim.x + threadIdx.x, de = gridDim.x * blockDim.x;
+  const int nx = (T_max + 1) * n, nu = T_max * m, nk = nu * n;
+  for (int b = blockIdx.y; b < B; b += gridDim.y) {
+    double* Xb = X ? X + (long long)b * nx : nullptr;
+    double* Ub = U ? U + (long long)b * nu : nullptr;
+    double* Vb = Vx ? Vx + (long long)b * nx : nullptr;
+    double* Kb = K ? K + (long long)b * nk : nullptr;
     if (rejected) {
-      if (X) for (int i = 0; i < n; ++i) X[t * n + i] = qnan;
-      if (U && k < T_max) for (int i = 0; i < m; ++i) U[((long long)b * T_max + k) * m + i] = qnan;
-      if (Vx) for (int i = 0; i < n; ++i) Vx[t * n + i] = qnan;
-      if (K && k < T_max) for (int i = 0; i < m * n; ++i) K[((long long)b * T_max + k) * m * n + i] = qnan;
+      if (X) for (int e = e0; e < nx; e += de) Xb[e] = qnan;
+      if (U) for (int e = e0; e < nu; e += de) Ub[e] = qnan;
+      if (Vx) for (int e = e0; e < nx; e += de) Vb[e] = qnan;
+      if (K) for (int e = e0; e < nk; e += de) Kb[e] = qnan;
       continue;
     }
     const int Tb = min(max(T[b], 0), T_max);
     const long long base = toff[b];
     const int sl = min(max(slot[b], 0), NS - 1);
-    const long long xr = ((base + min(k, Tb)) * NS + sl) * RS;
     auto rd = [&](const void* p, long long idx) -> double {
       return rbytes == 8 ? reinterpret_cast<const double*>(p)[idx] : (double)reinterpret_cast<const float*>(p)[idx];
     };
     if (X)   // float32 records carry the state's low parts after u
-      for (int i = 0; i < n; ++i) X[t * n + i] = rd(traj, xr + i) + (rbytes == 4 ? rd(traj, xr + n + m + i) : 0.0);
-    if (U && k < T_max)
-      for (int i = 0; i < m; ++i)
-        U[((long long)b * T_max + k) * m + i] = k < Tb ? rd(traj, ((base + k) * NS + sl) * RS + n + i) : 0.0;
+      for (int e = rows_done ? (Tb + 1) * n + e0 : e0; e < nx; e += de) {
+        const int k = min(e / n, Tb), i = e % n;
+        const long long xr = ((base + k) * NS + sl) * RS;
+        Xb[e] = rd(traj, xr + i) + (rbytes == 4 ? rd(traj, xr + n + m + i) : 0.0);
+      }
+    if (U)
+      for (int e = rows_done ? Tb * m + e0 : e0; e < nu; e += de) {
+        const int k = e / m;
+        Ub[e] = k < Tb ? rd(traj, ((base + k) * NS + sl) * RS + n + e % m) : 0.0;
+      }
     if (Vx)
-      for (int i = 0; i < n; ++i) Vx[t * n + i] = (vx && k <= Tb) ? vx[(base + k) * n + i] : 0.0;
-    if (K && k < T_max)
-      for (int i = 0; i < m * n; ++i)
-        K[((long long)b * T_max + k) * m * n + i] = k < Tb ? rd(gains, (base + k) * GS + i) : 0.0;
+      for (int e = e0; e < nx; e += de) Vb[e] = (vx && e / n <= Tb) ? vx[base * n + e] : 0.0;
+    if (K)
+      for (int e = e0; e < nk; e += de) {
+        const int k = e / (m * n);
+        Kb[e] = k < Tb ? rd(gains, (base + k) * GS + e % (m * n)) : 0.0;
+      }
   }
+}
+
+// the gather's grid for B instances whose longest output has this many
+// elements: 4 elements a thread
+static dim3 gather_grid(int B, int elems) {
+  return dim3(std::max(1, (elems + 1023) / 1024), (unsigned)std::min(B, 65535));
 }
 
 // Vbar_k = sum_{j=k}^{min(k+K,T)-1} l_j + [k + K >= T] l_T over the per-knot
@@ -547,6 +570,8 @@ static int launch_solve(to_batch b, int B, const double* d_x0, const int* d_T, c
                                       b->queue, b->J, b->iters);
     TO_CK(cudaGetLastError());
   }
+  b->rows_done = !serve && b->X_out && ops->rows_out && G > 1;
+  if (b->rows_done) { a.X_out = b->X_out; a.U_out = b->U_out; }
   TO_CK(ops->launch(prec, G, depth, gpb, grid, s, a));
   b->B = B;
   b->max_iter = o->max_iter;
@@ -568,13 +593,9 @@ int to_resolve_shape(to_problem p, const to_solver_opts* o, int B, double frac, 
   return resolve_shape(p, o, B, frac, G, gpb, grid, bps, depth);
 }
 
-int to_ensure_workspace(to_batch b, const to_solver_opts* o, bool want_traj) {
+int to_ensure_workspace(to_batch b, const to_solver_opts* o) {
   int rc = ensure_options(b, o, false, false);
   if (rc) return rc;
-  to_problem p = b->p;
-  size_t dummy = 0;
-  if (want_traj && !b->gX) TO_CK(grow(b->gX, (size_t)b->B_max * (p->T_max + 1) * p->n, dummy));
-  if (want_traj && !b->gU) TO_CK(grow(b->gU, (size_t)b->B_max * p->T_max * p->m, dummy));
   return TO_OK;
 }
 
@@ -582,9 +603,9 @@ int to_enqueue_gather(to_batch b, int B, const int* d_T, double* d_X, double* d_
   to_problem p = b->p;
   const int pi = b->prec == TO_FP64 ? 0 : 1;
   const int NS = std::min(b->G, kLsWidth) + 1;
-  gather_kernel<<<1024, 256, 0, s>>>(B, p->T_max, p->n, p->m, p->ops->rs[pi], p->ops->gs[pi], NS, pi == 0 ? 8 : 4,
-                                     b->toff, d_T, b->slot, b->traj, b->gains, nullptr, d_X, d_U, nullptr, nullptr,
-                                     b->err);
+  gather_kernel<<<gather_grid(B, (p->T_max + 1) * p->n), 256, 0, s>>>(
+      B, p->T_max, p->n, p->m, p->ops->rs[pi], p->ops->gs[pi], NS, pi == 0 ? 8 : 4, b->toff, d_T, b->slot, b->traj,
+      b->gains, nullptr, d_X, d_U, nullptr, nullptr, b->err, b->rows_done);
   TO_CK(cudaGetLastError());
   return TO_OK;
 }
@@ -747,10 +768,9 @@ int toget_trajectories(to_batch b, double* X, double* U, double* J, int* iters, 
     const int rs = o->rs[rbytes == 8 ? 0 : 1], gs = o->gs[rbytes == 8 ? 0 : 1];
     (void)pi;
     const int NS = std::min(b->G, kLsWidth) + 1;
-    gather_kernel<<<1024, 256, 0, b->stream>>>(B, p->T_max, p->n, p->m, rs, gs, NS, rbytes, b->toff, b->last_T, b->slot,
-                                               b->traj,
-                                               b->gains, b->vx, X ? b->gX : nullptr, U ? b->gU : nullptr,
-                                               Vx ? b->gV : nullptr, K ? b->gK : nullptr, b->err);
+    gather_kernel<<<gather_grid(B, std::max((p->T_max + 1) * p->n, K ? p->T_max * p->m * p->n : 0)), 256, 0, b->stream>>>(
+        B, p->T_max, p->n, p->m, rs, gs, NS, rbytes, b->toff, b->last_T, b->slot, b->traj, b->gains, b->vx,
+        X ? b->gX : nullptr, U ? b->gU : nullptr, Vx ? b->gV : nullptr, K ? b->gK : nullptr, b->err, false);
     TO_CK(cudaGetLastError());
   }
   if (X) TO_CK(cudaMemcpyAsync(X, b->gX, nX * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
@@ -920,8 +940,9 @@ int tosolve_batch_noalloc(to_problem p, int B, const double* d_x0, const int* d_
   if (rc) return rc;
   if (d_X || d_U) {
     const int NS = std::min(w.G, kLsWidth) + 1;
-    gather_kernel<<<1024, 256, 0, s>>>(B, p->T_max, p->n, p->m, ops->rs[pi], ops->gs[pi], NS, elem, w.toff, d_T,
-                                       w.slot, w.traj, w.gains, nullptr, d_X, d_U, nullptr, nullptr, w.err);
+    gather_kernel<<<gather_grid(B, (p->T_max + 1) * p->n), 256, 0, s>>>(
+        B, p->T_max, p->n, p->m, ops->rs[pi], ops->gs[pi], NS, elem, w.toff, d_T, w.slot, w.traj, w.gains, nullptr,
+        d_X, d_U, nullptr, nullptr, w.err, false);
     TO_CK(cudaGetLastError());
   }
   return TO_OK;

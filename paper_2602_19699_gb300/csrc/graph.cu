@@ -139,7 +139,7 @@ int totune(to_problem p, int B, const double* x0, const int* T, to_solver_opts* 
   base.stage_depth = 0;
   rc = tocreate_batch(p, B, knots, &base, &w.b);
   if (rc) return rc;
-  rc = to_ensure_workspace(w.b, &base, false);
+  rc = to_ensure_workspace(w.b, &base);
   if (rc) return rc;
   GR_CK(cudaStreamCreateWithFlags(&w.s, cudaStreamNonBlocking));
   GR_CK(cudaEventCreate(&w.e0));
@@ -211,6 +211,8 @@ struct to_graph_s {
     double* J = nullptr;
     int* iters = nullptr;
     int* status = nullptr;
+    double* dX = nullptr;   // the device's addresses of X and U
+    double* dU = nullptr;
     cudaStream_t s = nullptr;
     cudaEvent_t done = nullptr;
   };
@@ -255,14 +257,15 @@ static int record_member(to_graph_s::Member& mm, const to_solver_opts* opts, dou
   GR_CK(cudaMemcpyAsync(b->x0, mm.x0, sizeof(double) * B * p->n, cudaMemcpyHostToDevice, mm.s));
   GR_CK(cudaMemcpyAsync(b->T, mm.T, sizeof(int) * B, cudaMemcpyHostToDevice, mm.s));
   b->grid_frac = frac;
+  b->X_out = mm.dX;
+  b->U_out = mm.dU;
   int rc = to_launch_core(b, B, b->x0, b->T, nullptr, nullptr, opts, mm.s, nullptr);
   b->grid_frac = 1.0;
+  b->X_out = b->U_out = nullptr;
   if (rc) return rc;
   if (want_traj) {
-    rc = to_enqueue_gather(b, B, b->T, b->gX, b->gU, mm.s);
+    rc = to_enqueue_gather(b, B, b->T, mm.dX, mm.dU, mm.s);
     if (rc) return rc;
-    GR_CK(cudaMemcpyAsync(mm.X, b->gX, sizeof(double) * B * (p->T_max + 1) * p->n, cudaMemcpyDeviceToHost, mm.s));
-    GR_CK(cudaMemcpyAsync(mm.U, b->gU, sizeof(double) * B * p->T_max * p->m, cudaMemcpyDeviceToHost, mm.s));
   }
   GR_CK(cudaMemcpyAsync(mm.J, b->J, sizeof(double) * B, cudaMemcpyDeviceToHost, mm.s));
   GR_CK(cudaMemcpyAsync(mm.iters, b->iters, sizeof(int) * B, cudaMemcpyDeviceToHost, mm.s));
@@ -304,12 +307,14 @@ int tograph_create(const to_batch* batches, const int* B, const double* shares, 
     mm.b = batches[i];
     mm.B = B[i];
     to_problem p = mm.b->p;
-    rc = to_ensure_workspace(mm.b, opts, want_traj != 0);
+    rc = to_ensure_workspace(mm.b, opts);
     if (rc) return bail(rc);
     cudaError_t e = pinned(&mm.x0, (size_t)mm.B * p->n);
     if (e == cudaSuccess) e = pinned(&mm.T, (size_t)mm.B);
     if (e == cudaSuccess && want_traj) e = pinned(&mm.X, (size_t)mm.B * (p->T_max + 1) * p->n);
     if (e == cudaSuccess && want_traj) e = pinned(&mm.U, (size_t)mm.B * p->T_max * p->m);
+    if (e == cudaSuccess && want_traj) e = cudaHostGetDevicePointer((void**)&mm.dX, mm.X, 0);
+    if (e == cudaSuccess && want_traj) e = cudaHostGetDevicePointer((void**)&mm.dU, mm.U, 0);
     if (e == cudaSuccess) e = pinned(&mm.J, (size_t)mm.B);
     if (e == cudaSuccess) e = pinned(&mm.iters, (size_t)mm.B);
     if (e == cudaSuccess) e = pinned(&mm.status, (size_t)mm.B);

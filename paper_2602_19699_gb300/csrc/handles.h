@@ -62,6 +62,11 @@ struct to_batch_s {
   double* gV = nullptr;
   double* gK = nullptr;
   unsigned long long* prof = nullptr;   // 8 per-phase cycle counters
+  // where the next solve may write X and U itself as each instance is done, up to its
+  // horizon (instance-major float64, device-visible), or null; rows_done: the last solve did
+  double* X_out = nullptr;
+  double* U_out = nullptr;
+  bool rows_done = false;
   // last solve
   int B = 0, max_iter = 0, prec = TO_MIXED, want_vx = 0, launches = 0, G = 8;
   const int* last_T = nullptr;
@@ -85,10 +90,11 @@ int to_check_opts(const to_solver_opts* o);
 int to_resolve_shape(to_problem p, const to_solver_opts* o, int B, double frac, int* G, int* gpb, int* grid,
                      int* ctas_per_sm, int* depth = nullptr);
 
-// grow the option-dependent workspace (per-iteration history; with
-// want_traj, the X / U gather staging) so that a solve allocates nothing
-int to_ensure_workspace(to_batch b, const to_solver_opts* o, bool want_traj);
+// grow the option-dependent workspace (per-iteration history) so that a
+// solve allocates nothing
+int to_ensure_workspace(to_batch b, const to_solver_opts* o);
 
 // gather the last solve's X (B x (T_max+1) x n) and U (B x T_max x m) as
-// float64 into device buffers (either may be null) on stream s
+// float64 into device-visible buffers (either may be null) on stream s: the
+// padding only where the solve has written its rows there (rows_done)
 int to_enqueue_gather(to_batch b, int B, const int* d_T, double* d_X, double* d_U, cudaStream_t s);

@@ -86,6 +86,8 @@ struct SolveArgs {
   void* traj;               // knot records [x | u | pad] (R), (LW + 1) slots per knot
   void* gains;              // gain records [K (m x n) | k (m) | pad] (R)
   double* vx;               // knots x n, or null
+  double* X_out;            // B x (T_max + 1) x n: rows up to the horizon, or null (see writes_rows)
+  double* U_out;            // B x T_max x m
   double* J_out;
   int* iters_out;
   int* status_out;
@@ -227,6 +229,12 @@ enum { M_IDLE = 0, M_NEW, M_RUN, M_FINAL, M_DRAINED };
 // (and the backward pass is redone), divided by it after an accepted step
 // (not below kMuMin); beyond kMuMax the instance stops with LS_FAIL
 constexpr double kMu0 = 1e-6, kMuMin = 1e-8, kMuMax = 1e10, kMuFactor = 10.0;
+
+// Does a group write its returned iterate out itself (SolveArgs.X_out)?  Not
+// single lanes (their stores would be scattered), and not the rigid trees,
+// whose solve is long beside the copy: the code alone took the 7-DoF arm
+// (B = 2048, T = 50 to 200) from 16.9 to 18.1 ms.
+template <class Sys> constexpr bool writes_rows(int G) { return G > 1 && !Sys::kKnotParallel; }
 
 // D is the staging depth: a group fetches the records it will read D knots
 // ahead of the knot that reads them (the backward pass's knot record or
@@ -1462,6 +1470,26 @@ struct Solver {
     }
   }
 
+  // The returned iterate as instance-major float64 rows, written by the group
+  // that solved it as soon as it is done: straight into a captured solve's
+  // pinned staging, over the link to the host while other groups still solve.
+  // Gathered and copied after the solve, 237 MB (planar arm, B = 8192, T = 100
+  // to 400, 5 iterations) took 15.85 ms instead of 15.48, 24 MB (car, B = 8192,
+  // T = 20 to 50) 0.734 instead of 0.699; a gather into the staging without
+  // these rows was no faster than the copy.
+  TO_DEV static void put_rows(const Group<G>& g, const SolveArgs& a, R* traj, long long base, int T, int cur,
+                              int inst) {
+    double* X = a.X_out + (long long)inst * (a.T_max + 1) * n;
+    double* U = a.U_out + (long long)inst * a.T_max * m;
+#pragma unroll 4
+    for (int e = g.lane; e < (T + 1) * n; e += G) {
+      const R* r = rec(a, traj, base, e / n, cur);
+      X[e] = (double)r[e % n] + (kLo ? (double)r[n + m + e % n] : 0.0);
+    }
+#pragma unroll 4
+    for (int e = g.lane; e < T * m; e += G) U[e] = (double)rec(a, traj, base, e / m, cur)[n + e % m];
+  }
+
   // ------------------------------------------------------------------------
   // the kernel body
   // ------------------------------------------------------------------------
@@ -1938,6 +1966,9 @@ struct Solver {
         }
       }
       if (release) {
+        if constexpr (writes_rows<Sys>(G)) {
+          if (a.X_out) put_rows(g, a, traj, base, T, cur, inst);
+        }
         if (g.lane == 0) {
           a.J_out[inst] = J;
           a.iters_out[inst] = iter;
@@ -1969,6 +2000,7 @@ __global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, in
                               const int* __restrict__ slot,
                               const void* __restrict__ traj, const void* __restrict__ gains,
                               const double* __restrict__ vx, double* __restrict__ X, double* __restrict__ U,
-                              double* __restrict__ Vx, double* __restrict__ K, const int* __restrict__ err);
+                              double* __restrict__ Vx, double* __restrict__ K, const int* __restrict__ err,
+                              bool rows_done);
 
 }  // namespace to

@@ -32,6 +32,7 @@ struct SysOps {
   // result does not depend on the batch it is solved in), and each other
   // size's CTAs have 64 threads
   int (*lanes)(int prec, int B, int sms);
+  bool rows_out;                    // its groups of more than one lane write SolveArgs.X_out
   bool accepts_actor;
   // parse the flat parameter vector into the system's struct in float64 and float32
   int (*parse)(const double* p, size_t np, std::vector<unsigned char>& blob64, std::vector<unsigned char>& blob32,
@@ -195,6 +196,7 @@ inline void fill_layout(SysOps& o) {
   o.gs[0] = Layout<Sys, double>::GS;
   o.rs[1] = Layout<Sys, float>::RS;
   o.gs[1] = Layout<Sys, float>::GS;
+  o.rows_out = writes_rows<Sys>(2);
 }
 
 // shared checks of the rigid-body parameter format (see include/to.h)
