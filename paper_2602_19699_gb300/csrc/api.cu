@@ -122,9 +122,11 @@ __global__ void prepare_kernel(int B, const int* __restrict__ T, int T_max, long
 //
 // Bound by memory.  A block takes an instance (grid.y) and a stretch of its
 // output elements, one thread each, so that every store and, within a record,
-// every load is of consecutive addresses (one thread per knot, as before,
-// stored 8 bytes every 48).  rows_done: the solver has written the rows up to
-// the horizon (SolveArgs.X_out, U_out), the padding remains.
+// every load is of consecutive addresses (a thread per knot stored 8
+// bytes every 48, and read a quadruped's 432 gains alone: reading back those
+// gains, B = 512, T = 8, took 236 us and takes 137).  rows_done: the solver has
+// written the rows up to the horizon (SolveArgs.X_out, U_out), the padding
+// remains.
 __global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, int NS, int rbytes,
                               const long long* __restrict__ toff, const int* __restrict__ T,
                               const int* __restrict__ slot,
@@ -338,7 +340,7 @@ void todestroy_problem(to_problem p) {
 static void free_batch_buffers(to_batch b) {
   void* ptrs[] = {b->x0, b->T, b->U_init, b->forced, b->toff, b->order, b->hist, b->err, b->queue, b->traj,
                   b->gains, b->dscr, b->vx, b->J, b->iters, b->status, b->slot, b->ahist, b->Jhist, b->gX, b->gU,
-                  b->gV, b->gK, b->prof};
+                  b->gV, b->gK, b->gC, b->prof};
   for (void* q : ptrs)
     if (q) cudaFree(q);
 }
@@ -792,8 +794,15 @@ int toget_critic_targets(to_batch b, int K, double* Vbar) {
   if (B == 0) return TO_OK;
   if (!b->last_T) return fail(TO_ERR_ARG, "toget_critic_targets: the batch holds no solve");
   const size_t cnt = (size_t)B * (p->T_max + 1);
-  double* d = nullptr;
-  TO_CK(cudaMalloc(&d, 2 * cnt * sizeof(double)));
+  // kept by the batch: an allocation and a release a call were most of its 190
+  // us (B = 2048, T = 100)
+  if (b->gC_cap < cnt) {
+    size_t dummy = 0;
+    b->gC_cap = 0;
+    TO_CK(grow(b->gC, 2 * cnt, dummy));
+    b->gC_cap = cnt;
+  }
+  double* d = b->gC;
   KnotCostArgs ka{};
   ka.B = B;
   ka.T_max = p->T_max;
@@ -813,7 +822,6 @@ int toget_critic_targets(to_batch b, int K, double* Vbar) {
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(Vbar, d + cnt, cnt * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  cudaFree(d);
   if (e != cudaSuccess) return fail(TO_ERR_CUDA, std::string("toget_critic_targets: ") + cudaGetErrorString(e));
   return TO_OK;
 }

@@ -61,6 +61,9 @@ struct to_batch_s {
   double* gU = nullptr;
   double* gV = nullptr;
   double* gK = nullptr;
+  // critic targets: per-knot costs and windows of the largest batch asked for so far
+  double* gC = nullptr;
+  size_t gC_cap = 0;
   unsigned long long* prof = nullptr;   // 8 per-phase cycle counters
   // where the next solve may write X and U itself as each instance is done, up to its
   // horizon (instance-major float64, device-visible), or null; rows_done: the last solve did
