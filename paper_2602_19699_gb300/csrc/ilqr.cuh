@@ -1699,8 +1699,16 @@ struct Solver {
               for (int i = g.lane; i < n; i += G) vx_at(a, a.vx, base + T)[i] = (double)w.v[i];
             // (one lane used to rewrite the constant Hessians at every knot)
             if (bw) Sys::running_consts(P, g.lane, G, (R)a.eps, w.lxx, w.lx, w.luu);
-            // every lane: the substep primal chains of its knots (bw is uniform over a group of whole warps)
-            if (bw)
+            // the knots' substep primals (bw is uniform over a group of whole warps): by the
+            // group, or every lane the chains of its knots
+            bool chains = bw;
+            if constexpr (Sys::template kGroupStep<G>)
+              if (bw && P.free_base) {      // uniform over the grid
+                Sys::template primals_group<R, G>(P, g, T, [&](int k) { return rec(a, traj, base, k, cur); },
+                                                  [&](int k) { return dscr_at(a, base + k); }, w.sx);
+                chains = false;
+              }
+            if (chains)
               for (int k = g.lane; k < T; k += G) {
                 const R* r = rec(a, traj, base, k, cur);
                 R x[n], u[m];

@@ -805,10 +805,292 @@ struct SysRigid {
     cross_acc(vw, hf, ff);
   }
 
+  // a knot's substeps by its team, from the state and the joint torques in its
+  // slot, where the new state is left; prims (nullable): the state and the
+  // accelerations of every substep are put into the knot's stored Prims
+  template <class R, int G>
+  TO_DEV static void team_steps(const ParamsT<R>& P, bool on, R* slot, int sub, R* prims) {
+    constexpr int TL = G / kStepSlots, LP = 4 / TL;
+    R bq[6], bql[6], bv[6], bvl[6], lq[LP][3], lql[LP][3], lv[LP][3], lvl[LP][3], tau[LP][3];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) { bq[i] = slot[i]; bql[i] = slot[n + i]; bv[i] = slot[N + i]; bvl[i] = slot[n + N + i]; }
+#pragma unroll
+    for (int p = 0; p < LP; ++p)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int j = 3 * (sub * LP + p) + k;
+        lq[p][k] = slot[6 + j]; lql[p][k] = slot[n + 6 + j];
+        lv[p][k] = slot[N + 6 + j]; lvl[p][k] = slot[n + N + 6 + j];
+        tau[p][k] = slot[2 * n + j];
+      }
+    const R h = P.dt / (R)P.n_sub, ib = R(1) / P.beta;
+    for (int st = 0; st < P.n_sub; ++st) {
+      if (prims && on) {
+        Prim<R>& pr = *reinterpret_cast<Prim<R>*>(prims + (size_t)st * kPrimStride<R>);
+        if (sub == 0)
+#pragma unroll
+          for (int i = 0; i < 6; ++i) { pr.q[i] = bq[i]; pr.qd[i] = bv[i]; }
+#pragma unroll
+        for (int p = 0; p < LP; ++p)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            const int j = 6 + 3 * (sub * LP + p) + k;
+            pr.q[j] = lq[p][k]; pr.qd[j] = lv[p][k]; pr.tin[j] = tau[p][k];
+          }
+      }
+      // the base: E0 maps world to body axes
+      R sz, cz, sy, cy, sx, cx;
+      dsincos(bq[3], &sz, &cz);
+      dsincos(bq[4], &sy, &cy);
+      dsincos(bq[5], &sx, &cx);
+      const R E0[9] = {cy * cz,                cy * sz,                -sy,
+                       sx * sy * cz - cx * sz, sx * sy * sz + cx * cz, sx * cy,
+                       cx * sy * cz + sx * sz, cx * sy * sz - sx * cz, cx * cy};
+      R w[3], v[3], aw[3], av[3], fb[3], nb[3];
+      const R dz = bv[3], dy = bv[4], dx = bv[5], zy = dz * dy;
+      w[0] = dx - sy * dz; w[1] = cx * dy + sx * cy * dz; w[2] = cx * cy * dz - sx * dy;
+      aw[0] = -cy * zy; aw[1] = w[2] * dx - sx * sy * zy; aw[2] = -(w[1] * dx) - cx * sy * zy;
+      mv(E0, bv, v);
+      mv(E0, P.g, av);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) av[k] = -av[k];
+      cross_acc(v, w, av);
+      // sums over the legs: the 6 x 6 matrix (lower, rows n then f) and the right-hand side
+      R S[21], y[6];
+      {
+        R hn[3], hf[3];
+        inertia_mul(P, 5, aw, av, nb, fb);
+        inertia_mul(P, 5, w, v, hn, hf);
+        cross_acc(w, hn, nb);
+        cross_acc(v, hf, nb);
+        cross_acc(w, hf, fb);
+      }
+#pragma unroll
+      for (int i = 0; i < 21; ++i) S[i] = R(0);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) y[i] = R(0);
+      R mc = R(0), hc[3] = {R(0), R(0), R(0)}, Ic[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
+      R F[LP][3][6], yr[LP][3], l00[LP], l10[LP], l20[LP], l11[LP], l21[LP], l22[LP];
+#pragma unroll
+      for (int p = 0; p < LP; ++p) {
+        const int leg = sub * LP + p, bi = 6 + 3 * leg;
+        R s0, c0, s1, c1, s2, c2;
+        dsincos(lq[p][0], &s0, &c0);
+        dsincos(lq[p][1], &s1, &c1);
+        dsincos(lq[p][2], &s2, &c2);
+        const R* r0 = P.off[bi];
+        const R* r1 = P.off[bi + 1];
+        const R* r2 = P.off[bi + 2];
+        R w0[3], v0[3], a0[3], b0[3], n0[3], f0[3], w1[3], v1[3], a1[3], b1[3], n1[3], f1[3], w2[3], v2[3], a2[3], b2[3],
+            n2[3], f2[3];
+        leg_body<0>(P, bi, c0, s0, r0, lv[p][0], w, v, aw, av, w0, v0, a0, b0, n0, f0);
+        leg_body<1>(P, bi + 1, c1, s1, r1, lv[p][1], w0, v0, a0, b0, w1, v1, a1, b1, n1, f1);
+        leg_body<1>(P, bi + 2, c2, s2, r2, lv[p][2], w1, v1, a1, b1, w2, v2, a2, b2, n2, f2);
+        {  // contact at the foot: height and velocity in world axes, the force back in the calf's
+          const R pt[3] = {P.foot_pt[leg][0], P.foot_pt[leg][1], P.foot_pt[leg][2]};
+          R t[3], q[3], vel[3], Fw[3];
+          rot_t<1>(c2, s2, pt, t);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) t[k] += r2[k];
+          rot_t<1>(c1, s1, t, q);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) q[k] += r1[k];
+          rot_t<0>(c0, s0, q, t);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) t[k] += r0[k];
+          const R bz = P.beta * (bq[2] + (E0[2] * t[0] + E0[5] * t[1] + E0[8] * t[2]));
+#pragma unroll
+          for (int k = 0; k < 3; ++k) t[k] = v2[k];
+          cross_acc(w2, pt, t);
+          rot_t<1>(c2, s2, t, q);
+          rot_t<1>(c1, s1, q, t);
+          rot_t<0>(c0, s0, t, q);
+          mtv(E0, q, vel);
+          R sp, gate;
+          if (bz >= R(0)) {
+            const R e = dexp(-bz);
+            sp = ib * dlog1p(e);
+            gate = e / (R(1) + e);
+          } else {
+            const R e = dexp(bz);
+            sp = ib * (dlog1p(e) - bz);
+            gate = R(1) / (R(1) + e);
+          }
+          const R dg = P.dc * gate;
+          Fw[0] = -(dg * vel[0]);
+          Fw[1] = -(dg * vel[1]);
+          Fw[2] = P.kc * sp - dg * vel[2];
+          mv(E0, Fw, q);
+          rot<0>(c0, s0, q, t);
+          rot<1>(c1, s1, t, q);
+          rot<1>(c2, s2, q, t);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) f2[k] -= t[k];
+          cross_sub(pt, t, n2);
+        }
+        // bias torques, and the leg's wrench on the base
+        R rhs[3], nu[3], fu[3];
+        rhs[2] = tau[p][2] - n2[1];
+        force_up<1>(c2, s2, r2, n2, f2, nu, fu);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { n1[k] += nu[k]; f1[k] += fu[k]; }
+        rhs[1] = tau[p][1] - n1[1];
+        force_up<1>(c1, s1, r1, n1, f1, nu, fu);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { n0[k] += nu[k]; f0[k] += fu[k]; }
+        rhs[0] = tau[p][0] - n0[0];
+        force_up<0>(c0, s0, r0, n0, f0, nu, fu);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { y[k] -= nu[k]; y[3 + k] -= fu[k]; }
+        // composite inertias and joint columns (I e, e x h), carried to the base
+        R H00, H10, H20, H11, H21, H22;
+        {
+          R m2, h2[3], I2[6], m1, h1[3], I1[6], m0, h0[3], I0[6], n_[3], f_[3];
+          body_inertia(P, bi + 2, m2, h2, I2);
+          body_inertia(P, bi + 1, m1, h1, I1);
+          body_inertia(P, bi, m0, h0, I0);
+          inertia_up<1>(c2, s2, r2, m2, h2, I2, m1, h1, I1);
+          inertia_up<1>(c1, s1, r1, m1, h1, I1, m0, h0, I0);
+          inertia_up<0>(c0, s0, r0, m0, h0, I0, mc, hc, Ic);
+          const R cn[3] = {I2[3], I2[1], I2[5]}, cf[3] = {h2[2], R(0), -h2[0]};
+          H22 = I2[1];
+          force_up<1>(c2, s2, r2, cn, cf, n_, f_);
+          H21 = n_[1];
+          force_up<1>(c1, s1, r1, n_, f_, nu, fu);
+          H20 = nu[0];
+          force_up<0>(c0, s0, r0, nu, fu, &F[p][2][0], &F[p][2][3]);
+          const R tn[3] = {I1[3], I1[1], I1[5]}, tf[3] = {h1[2], R(0), -h1[0]};
+          H11 = I1[1];
+          force_up<1>(c1, s1, r1, tn, tf, nu, fu);
+          H10 = nu[0];
+          force_up<0>(c0, s0, r0, nu, fu, &F[p][1][0], &F[p][1][3]);
+          const R xn[3] = {I0[0], I0[3], I0[4]}, xf[3] = {R(0), -h0[2], h0[1]};
+          H00 = I0[0];
+          force_up<0>(c0, s0, r0, xn, xf, &F[p][0][0], &F[p][0][3]);
+        }
+        // H = L L^T (reciprocal diagonal); F <- L^-1 F^T, yr = L^-1 rhs
+        l00[p] = rsqrt_(H00);
+        l10[p] = H10 * l00[p];
+        l20[p] = H20 * l00[p];
+        l11[p] = rsqrt_(H11 - l10[p] * l10[p]);
+        l21[p] = (H21 - l20[p] * l10[p]) * l11[p];
+        l22[p] = rsqrt_(H22 - l20[p] * l20[p] - l21[p] * l21[p]);
+        yr[p][0] = rhs[0] * l00[p];
+        yr[p][1] = (rhs[1] - l10[p] * yr[p][0]) * l11[p];
+        yr[p][2] = (rhs[2] - l20[p] * yr[p][0] - l21[p] * yr[p][1]) * l22[p];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+          F[p][0][j] *= l00[p];
+          F[p][1][j] = (F[p][1][j] - l10[p] * F[p][0][j]) * l11[p];
+          F[p][2][j] = (F[p][2][j] - l20[p] * F[p][0][j] - l21[p] * F[p][1][j]) * l22[p];
+        }
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+#pragma unroll
+          for (int j = 0; j <= i; ++j)
+            S[i * (i + 1) / 2 + j] -= F[p][0][i] * F[p][0][j] + F[p][1][i] * F[p][1][j] + F[p][2][i] * F[p][2][j];
+          y[i] -= F[p][0][i] * yr[p][0] + F[p][1][i] * yr[p][1] + F[p][2][i] * yr[p][2];
+        }
+      }
+      // the legs' composite inertia in spatial form: n = I a + h x b, f = m b - h x a
+      S[0] += Ic[0]; S[2] += Ic[1]; S[5] += Ic[2]; S[1] += Ic[3]; S[3] += Ic[4]; S[4] += Ic[5];
+      S[9] += mc; S[14] += mc; S[20] += mc;
+      S[7] += hc[2]; S[8] -= hc[1]; S[10] -= hc[2]; S[12] += hc[0]; S[15] += hc[1]; S[16] -= hc[0];
+#pragma unroll
+      for (int o = 1; o < TL; o <<= 1) {
+#pragma unroll
+        for (int i = 0; i < 21; ++i) S[i] += __shfl_xor_sync(0xffffffffu, S[i], o);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) y[i] += __shfl_xor_sync(0xffffffffu, y[i], o);
+      }
+      {  // the base body itself
+        R m5, h5[3], I5[6];
+        body_inertia(P, 5, m5, h5, I5);
+        S[0] += I5[0]; S[2] += I5[1]; S[5] += I5[2]; S[1] += I5[3]; S[3] += I5[4]; S[4] += I5[5];
+        S[9] += m5; S[14] += m5; S[20] += m5;
+        S[7] += h5[2]; S[8] -= h5[1]; S[10] -= h5[2]; S[12] += h5[0]; S[15] += h5[1]; S[16] -= h5[0];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { y[k] -= nb[k]; y[3 + k] -= fb[k]; }
+      }
+      // a_b: Cholesky of the 6 x 6 (reciprocal diagonal), two triangular solves
+#pragma unroll
+      for (int j = 0; j < 6; ++j) {
+        R d = S[j * (j + 1) / 2 + j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) d -= S[j * (j + 1) / 2 + k] * S[j * (j + 1) / 2 + k];
+        const R rd = rsqrt_(d);
+        S[j * (j + 1) / 2 + j] = rd;
+#pragma unroll
+        for (int i = j + 1; i < 6; ++i) {
+          R t = S[i * (i + 1) / 2 + j];
+#pragma unroll
+          for (int k = 0; k < j; ++k) t -= S[i * (i + 1) / 2 + k] * S[j * (j + 1) / 2 + k];
+          S[i * (i + 1) / 2 + j] = t * rd;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+#pragma unroll
+        for (int k = 0; k < i; ++k) y[i] -= S[i * (i + 1) / 2 + k] * y[k];
+        y[i] *= S[i * (i + 1) / 2 + i];
+      }
+#pragma unroll
+      for (int i = 5; i >= 0; --i) {
+#pragma unroll
+        for (int k = i + 1; k < 6; ++k) y[i] -= S[k * (k + 1) / 2 + i] * y[k];
+        y[i] *= S[i * (i + 1) / 2 + i];
+      }
+      // joint accelerations: the legs' by back substitution, the base's from its axes
+#pragma unroll
+      for (int p = 0; p < LP; ++p) {
+        R z[3], a[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          z[k] = yr[p][k];
+#pragma unroll
+          for (int j = 0; j < 6; ++j) z[k] -= F[p][k][j] * y[j];
+        }
+        a[2] = z[2] * l22[p];
+        a[1] = (z[1] - l21[p] * a[2]) * l11[p];
+        a[0] = (z[0] - l10[p] * a[1] - l20[p] * a[2]) * l00[p];
+        semi_implicit2<R, 3>(lq[p], lql[p], lv[p], lvl[p], a, h);
+        if (prims && on) {
+          Prim<R>& pr = *reinterpret_cast<Prim<R>*>(prims + (size_t)st * kPrimStride<R>);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) pr.qdd[6 + 3 * (sub * LP + p) + k] = a[k];
+        }
+      }
+      R ba[6];
+      mtv(E0, y + 3, ba);
+      ba[3] = (sx * y[1] + cx * y[2]) / cy;
+      ba[4] = cx * y[1] - sx * y[2];
+      ba[5] = y[0] + sy * ba[3];
+      semi_implicit2<R, 6>(bq, bql, bv, bvl, ba, h);
+      if (prims && on && sub == 0) {
+        Prim<R>& pr = *reinterpret_cast<Prim<R>*>(prims + (size_t)st * kPrimStride<R>);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) { pr.qdd[i] = ba[i]; pr.tin[i] = R(0); }
+      }
+    }
+    if (on) {
+      if (sub == 0)
+#pragma unroll
+        for (int i = 0; i < 6; ++i) { slot[i] = bq[i]; slot[n + i] = bql[i]; slot[N + i] = bv[i]; slot[n + N + i] = bvl[i]; }
+#pragma unroll
+      for (int p = 0; p < LP; ++p)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const int j = 3 * (sub * LP + p) + k;
+          slot[6 + j] = lq[p][k]; slot[n + 6 + j] = lql[p][k];
+          slot[N + 6 + j] = lv[p][k]; slot[n + N + 6 + j] = lvl[p][k];
+        }
+    }
+  }
+
   template <class R, int G>
   TO_DEV static R cost_step_team(const ParamsT<R>& P, const Group<G>& g, bool mine, R* xh, R* xl, const R* u, R* scratch) {
     static_assert(kGroupStep<G> && (G == 32 || G == 64), "16 teams of 2 or 4 lanes");
-    constexpr int TL = G / kStepSlots, LP = 4 / TL;
+    constexpr int TL = G / kStepSlots;
     R* flag = scratch + kStepSlots * kTeamSlot;
     R l = R(0);
     if (mine) {
@@ -824,259 +1106,8 @@ struct SysRigid {
     const int cand = g.lane / TL, sub = g.lane % TL;
     const bool on = flag[cand] != R(0);
     R* slot = scratch + cand * kTeamSlot;
-    if (__any_sync(0xffffffffu, on)) {       // a warp's teams run together (their sums are shuffles)
-      R bq[6], bql[6], bv[6], bvl[6], lq[LP][3], lql[LP][3], lv[LP][3], lvl[LP][3], tau[LP][3];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) { bq[i] = slot[i]; bql[i] = slot[n + i]; bv[i] = slot[N + i]; bvl[i] = slot[n + N + i]; }
-#pragma unroll
-      for (int p = 0; p < LP; ++p)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const int j = 3 * (sub * LP + p) + k;
-          lq[p][k] = slot[6 + j]; lql[p][k] = slot[n + 6 + j];
-          lv[p][k] = slot[N + 6 + j]; lvl[p][k] = slot[n + N + 6 + j];
-          tau[p][k] = slot[2 * n + j];
-        }
-      const R h = P.dt / (R)P.n_sub, ib = R(1) / P.beta;
-      for (int st = 0; st < P.n_sub; ++st) {
-        // the base: E0 maps world to body axes
-        R sz, cz, sy, cy, sx, cx;
-        dsincos(bq[3], &sz, &cz);
-        dsincos(bq[4], &sy, &cy);
-        dsincos(bq[5], &sx, &cx);
-        const R E0[9] = {cy * cz,                cy * sz,                -sy,
-                         sx * sy * cz - cx * sz, sx * sy * sz + cx * cz, sx * cy,
-                         cx * sy * cz + sx * sz, cx * sy * sz - sx * cz, cx * cy};
-        R w[3], v[3], aw[3], av[3], fb[3], nb[3];
-        const R dz = bv[3], dy = bv[4], dx = bv[5], zy = dz * dy;
-        w[0] = dx - sy * dz; w[1] = cx * dy + sx * cy * dz; w[2] = cx * cy * dz - sx * dy;
-        aw[0] = -cy * zy; aw[1] = w[2] * dx - sx * sy * zy; aw[2] = -(w[1] * dx) - cx * sy * zy;
-        mv(E0, bv, v);
-        mv(E0, P.g, av);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) av[k] = -av[k];
-        cross_acc(v, w, av);
-        // sums over the legs: the 6 x 6 matrix (lower, rows n then f) and the right-hand side
-        R S[21], y[6];
-        {
-          R hn[3], hf[3];
-          inertia_mul(P, 5, aw, av, nb, fb);
-          inertia_mul(P, 5, w, v, hn, hf);
-          cross_acc(w, hn, nb);
-          cross_acc(v, hf, nb);
-          cross_acc(w, hf, fb);
-        }
-#pragma unroll
-        for (int i = 0; i < 21; ++i) S[i] = R(0);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) y[i] = R(0);
-        R mc = R(0), hc[3] = {R(0), R(0), R(0)}, Ic[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-        R F[LP][3][6], yr[LP][3], l00[LP], l10[LP], l20[LP], l11[LP], l21[LP], l22[LP];
-#pragma unroll
-        for (int p = 0; p < LP; ++p) {
-          const int leg = sub * LP + p, bi = 6 + 3 * leg;
-          R s0, c0, s1, c1, s2, c2;
-          dsincos(lq[p][0], &s0, &c0);
-          dsincos(lq[p][1], &s1, &c1);
-          dsincos(lq[p][2], &s2, &c2);
-          const R* r0 = P.off[bi];
-          const R* r1 = P.off[bi + 1];
-          const R* r2 = P.off[bi + 2];
-          R w0[3], v0[3], a0[3], b0[3], n0[3], f0[3], w1[3], v1[3], a1[3], b1[3], n1[3], f1[3], w2[3], v2[3], a2[3], b2[3],
-              n2[3], f2[3];
-          leg_body<0>(P, bi, c0, s0, r0, lv[p][0], w, v, aw, av, w0, v0, a0, b0, n0, f0);
-          leg_body<1>(P, bi + 1, c1, s1, r1, lv[p][1], w0, v0, a0, b0, w1, v1, a1, b1, n1, f1);
-          leg_body<1>(P, bi + 2, c2, s2, r2, lv[p][2], w1, v1, a1, b1, w2, v2, a2, b2, n2, f2);
-          {  // contact at the foot: height and velocity in world axes, the force back in the calf's
-            const R pt[3] = {P.foot_pt[leg][0], P.foot_pt[leg][1], P.foot_pt[leg][2]};
-            R t[3], q[3], vel[3], Fw[3];
-            rot_t<1>(c2, s2, pt, t);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) t[k] += r2[k];
-            rot_t<1>(c1, s1, t, q);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) q[k] += r1[k];
-            rot_t<0>(c0, s0, q, t);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) t[k] += r0[k];
-            const R bz = P.beta * (bq[2] + (E0[2] * t[0] + E0[5] * t[1] + E0[8] * t[2]));
-#pragma unroll
-            for (int k = 0; k < 3; ++k) t[k] = v2[k];
-            cross_acc(w2, pt, t);
-            rot_t<1>(c2, s2, t, q);
-            rot_t<1>(c1, s1, q, t);
-            rot_t<0>(c0, s0, t, q);
-            mtv(E0, q, vel);
-            R sp, gate;
-            if (bz >= R(0)) {
-              const R e = dexp(-bz);
-              sp = ib * dlog1p(e);
-              gate = e / (R(1) + e);
-            } else {
-              const R e = dexp(bz);
-              sp = ib * (dlog1p(e) - bz);
-              gate = R(1) / (R(1) + e);
-            }
-            const R dg = P.dc * gate;
-            Fw[0] = -(dg * vel[0]);
-            Fw[1] = -(dg * vel[1]);
-            Fw[2] = P.kc * sp - dg * vel[2];
-            mv(E0, Fw, q);
-            rot<0>(c0, s0, q, t);
-            rot<1>(c1, s1, t, q);
-            rot<1>(c2, s2, q, t);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) f2[k] -= t[k];
-            cross_sub(pt, t, n2);
-          }
-          // bias torques, and the leg's wrench on the base
-          R rhs[3], nu[3], fu[3];
-          rhs[2] = tau[p][2] - n2[1];
-          force_up<1>(c2, s2, r2, n2, f2, nu, fu);
-#pragma unroll
-          for (int k = 0; k < 3; ++k) { n1[k] += nu[k]; f1[k] += fu[k]; }
-          rhs[1] = tau[p][1] - n1[1];
-          force_up<1>(c1, s1, r1, n1, f1, nu, fu);
-#pragma unroll
-          for (int k = 0; k < 3; ++k) { n0[k] += nu[k]; f0[k] += fu[k]; }
-          rhs[0] = tau[p][0] - n0[0];
-          force_up<0>(c0, s0, r0, n0, f0, nu, fu);
-#pragma unroll
-          for (int k = 0; k < 3; ++k) { y[k] -= nu[k]; y[3 + k] -= fu[k]; }
-          // composite inertias and joint columns (I e, e x h), carried to the base
-          R H00, H10, H20, H11, H21, H22;
-          {
-            R m2, h2[3], I2[6], m1, h1[3], I1[6], m0, h0[3], I0[6], n_[3], f_[3];
-            body_inertia(P, bi + 2, m2, h2, I2);
-            body_inertia(P, bi + 1, m1, h1, I1);
-            body_inertia(P, bi, m0, h0, I0);
-            inertia_up<1>(c2, s2, r2, m2, h2, I2, m1, h1, I1);
-            inertia_up<1>(c1, s1, r1, m1, h1, I1, m0, h0, I0);
-            inertia_up<0>(c0, s0, r0, m0, h0, I0, mc, hc, Ic);
-            const R cn[3] = {I2[3], I2[1], I2[5]}, cf[3] = {h2[2], R(0), -h2[0]};
-            H22 = I2[1];
-            force_up<1>(c2, s2, r2, cn, cf, n_, f_);
-            H21 = n_[1];
-            force_up<1>(c1, s1, r1, n_, f_, nu, fu);
-            H20 = nu[0];
-            force_up<0>(c0, s0, r0, nu, fu, &F[p][2][0], &F[p][2][3]);
-            const R tn[3] = {I1[3], I1[1], I1[5]}, tf[3] = {h1[2], R(0), -h1[0]};
-            H11 = I1[1];
-            force_up<1>(c1, s1, r1, tn, tf, nu, fu);
-            H10 = nu[0];
-            force_up<0>(c0, s0, r0, nu, fu, &F[p][1][0], &F[p][1][3]);
-            const R xn[3] = {I0[0], I0[3], I0[4]}, xf[3] = {R(0), -h0[2], h0[1]};
-            H00 = I0[0];
-            force_up<0>(c0, s0, r0, xn, xf, &F[p][0][0], &F[p][0][3]);
-          }
-          // H = L L^T (reciprocal diagonal); F <- L^-1 F^T, yr = L^-1 rhs
-          l00[p] = rsqrt_(H00);
-          l10[p] = H10 * l00[p];
-          l20[p] = H20 * l00[p];
-          l11[p] = rsqrt_(H11 - l10[p] * l10[p]);
-          l21[p] = (H21 - l20[p] * l10[p]) * l11[p];
-          l22[p] = rsqrt_(H22 - l20[p] * l20[p] - l21[p] * l21[p]);
-          yr[p][0] = rhs[0] * l00[p];
-          yr[p][1] = (rhs[1] - l10[p] * yr[p][0]) * l11[p];
-          yr[p][2] = (rhs[2] - l20[p] * yr[p][0] - l21[p] * yr[p][1]) * l22[p];
-#pragma unroll
-          for (int j = 0; j < 6; ++j) {
-            F[p][0][j] *= l00[p];
-            F[p][1][j] = (F[p][1][j] - l10[p] * F[p][0][j]) * l11[p];
-            F[p][2][j] = (F[p][2][j] - l20[p] * F[p][0][j] - l21[p] * F[p][1][j]) * l22[p];
-          }
-#pragma unroll
-          for (int i = 0; i < 6; ++i) {
-#pragma unroll
-            for (int j = 0; j <= i; ++j)
-              S[i * (i + 1) / 2 + j] -= F[p][0][i] * F[p][0][j] + F[p][1][i] * F[p][1][j] + F[p][2][i] * F[p][2][j];
-            y[i] -= F[p][0][i] * yr[p][0] + F[p][1][i] * yr[p][1] + F[p][2][i] * yr[p][2];
-          }
-        }
-        // the legs' composite inertia in spatial form: n = I a + h x b, f = m b - h x a
-        S[0] += Ic[0]; S[2] += Ic[1]; S[5] += Ic[2]; S[1] += Ic[3]; S[3] += Ic[4]; S[4] += Ic[5];
-        S[9] += mc; S[14] += mc; S[20] += mc;
-        S[7] += hc[2]; S[8] -= hc[1]; S[10] -= hc[2]; S[12] += hc[0]; S[15] += hc[1]; S[16] -= hc[0];
-#pragma unroll
-        for (int o = 1; o < TL; o <<= 1) {
-#pragma unroll
-          for (int i = 0; i < 21; ++i) S[i] += __shfl_xor_sync(0xffffffffu, S[i], o);
-#pragma unroll
-          for (int i = 0; i < 6; ++i) y[i] += __shfl_xor_sync(0xffffffffu, y[i], o);
-        }
-        {  // the base body itself
-          R m5, h5[3], I5[6];
-          body_inertia(P, 5, m5, h5, I5);
-          S[0] += I5[0]; S[2] += I5[1]; S[5] += I5[2]; S[1] += I5[3]; S[3] += I5[4]; S[4] += I5[5];
-          S[9] += m5; S[14] += m5; S[20] += m5;
-          S[7] += h5[2]; S[8] -= h5[1]; S[10] -= h5[2]; S[12] += h5[0]; S[15] += h5[1]; S[16] -= h5[0];
-#pragma unroll
-          for (int k = 0; k < 3; ++k) { y[k] -= nb[k]; y[3 + k] -= fb[k]; }
-        }
-        // a_b: Cholesky of the 6 x 6 (reciprocal diagonal), two triangular solves
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-          R d = S[j * (j + 1) / 2 + j];
-#pragma unroll
-          for (int k = 0; k < j; ++k) d -= S[j * (j + 1) / 2 + k] * S[j * (j + 1) / 2 + k];
-          const R rd = rsqrt_(d);
-          S[j * (j + 1) / 2 + j] = rd;
-#pragma unroll
-          for (int i = j + 1; i < 6; ++i) {
-            R t = S[i * (i + 1) / 2 + j];
-#pragma unroll
-            for (int k = 0; k < j; ++k) t -= S[i * (i + 1) / 2 + k] * S[j * (j + 1) / 2 + k];
-            S[i * (i + 1) / 2 + j] = t * rd;
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-#pragma unroll
-          for (int k = 0; k < i; ++k) y[i] -= S[i * (i + 1) / 2 + k] * y[k];
-          y[i] *= S[i * (i + 1) / 2 + i];
-        }
-#pragma unroll
-        for (int i = 5; i >= 0; --i) {
-#pragma unroll
-          for (int k = i + 1; k < 6; ++k) y[i] -= S[k * (k + 1) / 2 + i] * y[k];
-          y[i] *= S[i * (i + 1) / 2 + i];
-        }
-        // joint accelerations: the legs' by back substitution, the base's from its axes
-#pragma unroll
-        for (int p = 0; p < LP; ++p) {
-          R z[3], a[3];
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            z[k] = yr[p][k];
-#pragma unroll
-            for (int j = 0; j < 6; ++j) z[k] -= F[p][k][j] * y[j];
-          }
-          a[2] = z[2] * l22[p];
-          a[1] = (z[1] - l21[p] * a[2]) * l11[p];
-          a[0] = (z[0] - l10[p] * a[1] - l20[p] * a[2]) * l00[p];
-          semi_implicit2<R, 3>(lq[p], lql[p], lv[p], lvl[p], a, h);
-        }
-        R ba[6];
-        mtv(E0, y + 3, ba);
-        ba[3] = (sx * y[1] + cx * y[2]) / cy;
-        ba[4] = cx * y[1] - sx * y[2];
-        ba[5] = y[0] + sy * ba[3];
-        semi_implicit2<R, 6>(bq, bql, bv, bvl, ba, h);
-      }
-      if (on) {
-        if (sub == 0)
-#pragma unroll
-          for (int i = 0; i < 6; ++i) { slot[i] = bq[i]; slot[n + i] = bql[i]; slot[N + i] = bv[i]; slot[n + N + i] = bvl[i]; }
-#pragma unroll
-        for (int p = 0; p < LP; ++p)
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const int j = 3 * (sub * LP + p) + k;
-            slot[6 + j] = lq[p][k]; slot[n + 6 + j] = lql[p][k];
-            slot[N + 6 + j] = lv[p][k]; slot[n + N + 6 + j] = lvl[p][k];
-          }
-      }
-    }
+    // a warp's teams run together (their sums are shuffles)
+    if (__any_sync(0xffffffffu, on)) team_steps<R, G>(P, on, slot, sub, nullptr);
     g.sync();
     if (mine) {
       const R* s = scratch + g.lane * kTeamSlot;
@@ -1267,8 +1298,9 @@ struct SysRigid {
     R wpt[NF][3], F[NF][3], vb[NF][3], vwld[NF][3], gate[NF];
   };
   // Knot-parallel derivatives (both trees): before each backward pass every
-  // lane runs the substep primal chains of its own knots (primal_knot) and
-  // stores each substep's Prim in a per-knot global scratch; inside the
+  // lane runs the substep primal chains of its own knots (primal_knot; a
+  // free quadruped's group shares them, primals_group) and stores each
+  // substep's Prim in a per-knot global scratch; inside the
   // backward pass the group stages those Prims into shared memory
   // (cp.async, one substep ahead) and every direction lane runs its tangent
   // pass at once (derivs_staged).  No lane waits for a primal.
@@ -1711,6 +1743,54 @@ struct SysRigid {
     }
   }
 
+  template <class R> TO_DEV static void store_factor(Prim<R>& pr, const R* L) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      pr.L[k * N + k] = L[k * N + k];
+#pragma unroll
+      for (int d = 1; d <= kDepthMax; ++d)
+        if (d <= depth(k)) pr.L[k * N + anc(k, d)] = L[k * N + anc(k, d)];
+    }
+  }
+
+  // The stored primals of knots 0..T-1 by the whole group (a quadruped whose
+  // base is a free body): the substeps' states and accelerations by teams, 16
+  // knots at a time, then every substep's Prim by a lane of its own.  On one
+  // lane a knot's 10 substeps follow each other through 10 k instructions of
+  // straight-line code, and a short horizon fills a few lanes: a third of a
+  // solve.  B = 512 float32, 1 iteration with V_x: T = 4 to 8 6.60 -> 5.38 ms,
+  // T = 1 (device) 1.45 -> 0.75, T = 17 7.55 -> 7.28, T = 40 to 50 the same
+  // (21.8: the lanes were full).
+  template <class R, int G, class Rec, class Out>
+  TO_DEV static void primals_group(const ParamsT<R>& P, const Group<G>& g, int T, Rec rec, Out out, R* scratch) {
+    const int cand = g.lane / (G / kStepSlots), sub = g.lane % (G / kStepSlots);
+    for (int k0 = 0; k0 < T; k0 += kStepSlots) {
+      if (g.lane < kStepSlots && k0 + g.lane < T) {
+        const R* r = rec(k0 + g.lane);
+        R* s = scratch + g.lane * kTeamSlot;
+#pragma unroll
+        for (int i = 0; i < n; ++i) { s[i] = r[i]; s[n + i] = R(0); }
+#pragma unroll
+        for (int i = 0; i < m; ++i) s[2 * n + i] = r[n + i];
+      }
+      g.sync();
+      const bool on = k0 + cand < T;
+      if (__any_sync(0xffffffffu, on))
+        team_steps<R, G>(P, on, scratch + cand * kTeamSlot, sub, out(on ? k0 + cand : 0));
+      g.sync();
+    }
+    for (int e = g.lane; e < T * P.n_sub; e += G) {
+      Prim<R>& pr = *reinterpret_cast<Prim<R>*>(out(e / P.n_sub) + (size_t)(e % P.n_sub) * kPrimStride<R>);
+      R q[N], qd[N], hb[N], L[N * N], E[N][9], r[N][3];
+#pragma unroll
+      for (int i = 0; i < N; ++i) { q[i] = pr.q[i]; qd[i] = pr.qd[i]; }
+      bias_store(P, pr, q, qd, hb, E, r);
+      mass_chol(P, q, L, E, r);
+      store_factor(pr, L);
+      accel_store(P, pr);
+    }
+  }
+
   // The substep primal chain of one knot on one lane, every substep's Prim
   // stored at out + s kPrimStride (global memory): the same arithmetic as
   // derivs' primal lane, with the mass matrix factored on this lane.
@@ -1726,13 +1806,7 @@ struct SysRigid {
       bias_store(P, pr, q, qd, hb, E, r);
       if constexpr (kKeepBits<R>) mass_chol(P, q, L);
       else mass_chol(P, q, L, E, r);
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-        pr.L[k * N + k] = L[k * N + k];
-#pragma unroll
-        for (int d = 1; d <= kDepthMax; ++d)
-          if (d <= depth(k)) pr.L[k * N + anc(k, d)] = L[k * N + anc(k, d)];
-      }
+      store_factor(pr, L);
 #pragma unroll
       for (int i = 0; i < N; ++i) rhs[i] = tin[i] - hb[i];
       chol_solve(P, L, rhs, qdd);
