@@ -835,7 +835,8 @@ def config_legs(P, dev, flush, peak32, peak64, quad_budget=False):
                 wb = P.tocreate_batch(problem, B, B * (c["T"] + 1), wopts)
                 t_warm = _timed_solve(P, wb, B, d_x0[:B], d_T[:B], wopts, stream, flush, 1)
             ah, _ = P.toget_history(batch)
-            lanes = {W.POINTMASS: 8, W.ARM7: 16, W.QUAD: 16, W.DUBINS: 8}[sysid]   # step sizes per round
+            # step sizes per round (64 float64 point masses are solved 32 lanes each)
+            lanes = {W.POINTMASS: 16, W.ARM7: 16, W.QUAD: 16, W.DUBINS: 8}[sysid]
             alg = flops.solve_flops(prob.sys, prob.n, prob.m, b.T[:B], r["iters"], r["status"], ah,
                                     lanes_per_round=lanes, n_alpha=N_ALPHA, refine=prec == P.TO_MIXED,
                                     params=prob.params, actor=actor is not None)
