@@ -531,7 +531,7 @@ def run_gb300(args):
                        "oracle_self_reproducibility": dict(gates_self, perturbation="x0 * (1 +- 1e-15)")},
         "e2e": {"value": job_throughput(B * frac_mixed, e2e_max / args.steps, n), "unit": UNIT, "h2d_bytes_per_step": int(h2d),
                 "d2h_bytes_per_step": int(d2h), "ms_per_step": e2e_max / args.steps * 1e3,
-                "api": "tograph_launch of a captured solve (H2D from pinned staging, sort, solver, gather, D2H)",
+                "api": "tograph_launch of a captured solve (H2D from pinned staging, sort, solver with X and U written to pinned memory, padding, D2H)",
                 "kernels_per_step": int(e2e_launches), "results_equal_device_solve": e2e_same},
         "autotune": {"chosen": [int(opts.group_lanes), int(opts.groups_per_block), int(opts.stage_depth)],
                      "calibration": "the workload itself, max_iter=3",
