@@ -362,6 +362,9 @@ struct SysRigid {
     if (pa < 0) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) { Epw[k] = R(0); Ept[k] = R(0); aw[k] = R(0); t[k] = -P.g[k]; }
+      // (no force depends on where a sliding root stands: a non-finite position
+      // still ends in a non-finite cost)
+      if (jt > 2) t[ax] += R(0) * r[ax];
     } else {
       // X m = (E w, E (v - r x w))
 #pragma unroll
@@ -854,6 +857,9 @@ struct SysRigid {
       mv(E0, P.g, av);
 #pragma unroll
       for (int k = 0; k < 3; ++k) av[k] = -av[k];
+      // (no force depends on where the base stands in the plane: a non-finite
+      // position still ends in a non-finite cost)
+      av[0] += R(0) * bq[0] + R(0) * bq[1];
       cross_acc(v, w, av);
       // sums over the legs: the 6 x 6 matrix (lower, rows n then f) and the right-hand side
       R S[21], y[6];
