@@ -15,6 +15,7 @@
 #include <mutex>
 #include <vector>
 
+#include "gather_shape.h"
 #include "launch.cuh"
 #include "to.h"
 
@@ -126,7 +127,8 @@ __global__ void prepare_kernel(int B, const int* __restrict__ T, int T_max, long
 // bytes every 48, and read a quadruped's 432 gains alone: reading back those
 // gains, B = 512, T = 8, took 236 us and takes 137).  rows_done: the solver has
 // written the rows up to the horizon (SolveArgs.X_out, U_out), the padding
-// remains.
+// remains.  I: the type of an instance's element indices (gather_shape).
+template <class I>
 __global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, int NS, int rbytes,
                               const long long* __restrict__ toff, const int* __restrict__ T,
                               const int* __restrict__ slot,
@@ -136,18 +138,18 @@ __global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, in
                               bool rows_done) {
   const bool rejected = err && *err;
   const double qnan = __longlong_as_double(0x7ff8000000000000LL);
-  const int e0 = blockIdx.x * blockDim.x + threadIdx.x, de = gridDim.x * blockDim.x;
-  const int nx = (T_max + 1) * n, nu = T_max * m, nk = nu * n;
+  const I e0 = (I)blockIdx.x * blockDim.x + threadIdx.x, de = (I)gridDim.x * blockDim.x;
+  const I nx = ((I)T_max + 1) * n, nu = (I)T_max * m, nk = K ? nu * n : 0;
   for (int b = blockIdx.y; b < B; b += gridDim.y) {
     double* Xb = X ? X + (long long)b * nx : nullptr;
     double* Ub = U ? U + (long long)b * nu : nullptr;
     double* Vb = Vx ? Vx + (long long)b * nx : nullptr;
     double* Kb = K ? K + (long long)b * nk : nullptr;
     if (rejected) {
-      if (X) for (int e = e0; e < nx; e += de) Xb[e] = qnan;
-      if (U) for (int e = e0; e < nu; e += de) Ub[e] = qnan;
-      if (Vx) for (int e = e0; e < nx; e += de) Vb[e] = qnan;
-      if (K) for (int e = e0; e < nk; e += de) Kb[e] = qnan;
+      if (X) for (I e = e0; e < nx; e += de) Xb[e] = qnan;
+      if (U) for (I e = e0; e < nu; e += de) Ub[e] = qnan;
+      if (Vx) for (I e = e0; e < nx; e += de) Vb[e] = qnan;
+      if (K) for (I e = e0; e < nk; e += de) Kb[e] = qnan;
       continue;
     }
     const int Tb = min(max(T[b], 0), T_max);
@@ -157,30 +159,24 @@ __global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, in
       return rbytes == 8 ? reinterpret_cast<const double*>(p)[idx] : (double)reinterpret_cast<const float*>(p)[idx];
     };
     if (X)   // float32 records carry the state's low parts after u
-      for (int e = rows_done ? (Tb + 1) * n + e0 : e0; e < nx; e += de) {
-        const int k = min(e / n, Tb), i = e % n;
+      for (I e = rows_done ? ((I)Tb + 1) * n + e0 : e0; e < nx; e += de) {
+        const int k = (int)min(e / n, (I)Tb), i = (int)(e % n);
         const long long xr = ((base + k) * NS + sl) * RS;
         Xb[e] = rd(traj, xr + i) + (rbytes == 4 ? rd(traj, xr + n + m + i) : 0.0);
       }
     if (U)
-      for (int e = rows_done ? Tb * m + e0 : e0; e < nu; e += de) {
-        const int k = e / m;
+      for (I e = rows_done ? (I)Tb * m + e0 : e0; e < nu; e += de) {
+        const int k = (int)(e / m);
         Ub[e] = k < Tb ? rd(traj, ((base + k) * NS + sl) * RS + n + e % m) : 0.0;
       }
     if (Vx)
-      for (int e = e0; e < nx; e += de) Vb[e] = (vx && e / n <= Tb) ? vx[base * n + e] : 0.0;
+      for (I e = e0; e < nx; e += de) Vb[e] = (vx && e / n <= Tb) ? vx[base * n + e] : 0.0;
     if (K)
-      for (int e = e0; e < nk; e += de) {
-        const int k = e / (m * n);
+      for (I e = e0; e < nk; e += de) {
+        const int k = (int)(e / (m * n));
         Kb[e] = k < Tb ? rd(gains, (base + k) * GS + e % (m * n)) : 0.0;
       }
   }
-}
-
-// the gather's grid for B instances whose longest output has this many
-// elements: 4 elements a thread
-static dim3 gather_grid(int B, int elems) {
-  return dim3(std::max(1, (elems + 1023) / 1024), (unsigned)std::min(B, 65535));
 }
 
 // Vbar_k = sum_{j=k}^{min(k+K,T)-1} l_j + [k + K >= T] l_T over the per-knot
@@ -601,14 +597,21 @@ int to_ensure_workspace(to_batch b, const to_solver_opts* o) {
   return TO_OK;
 }
 
+cudaError_t to_gather(to_problem p, int prec_idx, int NS, int B, const long long* toff, const int* T, const int* slot,
+                      const void* traj, const void* gains, const double* vx, double* X, double* U, double* Vx, double* K,
+                      const int* err, bool rows_done, cudaStream_t s) {
+  const SysOps* o = p->ops;
+  const GatherShape g = gather_shape(B, gather_elems(p->T_max, p->n, p->m, K != nullptr));
+  auto* kernel = g.wide ? gather_kernel<long long> : gather_kernel<int>;
+  kernel<<<dim3(g.gx, g.gy), kGatherThreads, 0, s>>>(B, p->T_max, p->n, p->m, o->rs[prec_idx], o->gs[prec_idx], NS,
+                                                     prec_idx == 0 ? 8 : 4, toff, T, slot, traj, gains, vx, X, U, Vx, K,
+                                                     err, rows_done);
+  return cudaGetLastError();
+}
+
 int to_enqueue_gather(to_batch b, int B, const int* d_T, double* d_X, double* d_U, cudaStream_t s) {
-  to_problem p = b->p;
-  const int pi = b->prec == TO_FP64 ? 0 : 1;
-  const int NS = std::min(b->G, kLsWidth) + 1;
-  gather_kernel<<<gather_grid(B, (p->T_max + 1) * p->n), 256, 0, s>>>(
-      B, p->T_max, p->n, p->m, p->ops->rs[pi], p->ops->gs[pi], NS, pi == 0 ? 8 : 4, b->toff, d_T, b->slot, b->traj,
-      b->gains, nullptr, d_X, d_U, nullptr, nullptr, b->err, b->rows_done);
-  TO_CK(cudaGetLastError());
+  TO_CK(to_gather(b->p, b->prec == TO_FP64 ? 0 : 1, std::min(b->G, kLsWidth) + 1, B, b->toff, d_T, b->slot, b->traj,
+                  b->gains, nullptr, d_X, d_U, nullptr, nullptr, b->err, b->rows_done, s));
   return TO_OK;
 }
 
@@ -756,9 +759,6 @@ int toget_trajectories(to_batch b, double* X, double* U, double* J, int* iters, 
   TO_CK(cudaStreamSynchronize(b->stream));
   if (B == 0) return TO_OK;
   if ((Vx || K) && !b->want_vx) return fail(TO_ERR_ARG, "toget_trajectories: Vx / K need want_vx in the solve");
-  const SysOps* o = p->ops;
-  const int pi = b->elem_bytes == 8 && b->prec == TO_FP64 ? 0 : 1;
-  const int rbytes = b->prec == TO_FP64 ? 8 : 4;
   const size_t nX = (size_t)B * (p->T_max + 1) * p->n, nU = (size_t)B * p->T_max * p->m;
   const size_t nK = (size_t)B * p->T_max * p->m * p->n;
   size_t dummy = 0;
@@ -766,15 +766,10 @@ int toget_trajectories(to_batch b, double* X, double* U, double* J, int* iters, 
   if (U && !b->gU) TO_CK(grow(b->gU, (size_t)b->B_max * p->T_max * p->m, dummy));
   if (Vx && !b->gV) TO_CK(grow(b->gV, (size_t)b->B_max * (p->T_max + 1) * p->n, dummy));
   if (K && !b->gK) TO_CK(grow(b->gK, (size_t)b->B_max * p->T_max * p->m * p->n, dummy));
-  if (X || U || Vx || K) {
-    const int rs = o->rs[rbytes == 8 ? 0 : 1], gs = o->gs[rbytes == 8 ? 0 : 1];
-    (void)pi;
-    const int NS = std::min(b->G, kLsWidth) + 1;
-    gather_kernel<<<gather_grid(B, std::max((p->T_max + 1) * p->n, K ? p->T_max * p->m * p->n : 0)), 256, 0, b->stream>>>(
-        B, p->T_max, p->n, p->m, rs, gs, NS, rbytes, b->toff, b->last_T, b->slot, b->traj, b->gains, b->vx,
-        X ? b->gX : nullptr, U ? b->gU : nullptr, Vx ? b->gV : nullptr, K ? b->gK : nullptr, b->err, false);
-    TO_CK(cudaGetLastError());
-  }
+  if (X || U || Vx || K)
+    TO_CK(to_gather(p, b->prec == TO_FP64 ? 0 : 1, std::min(b->G, kLsWidth) + 1, B, b->toff, b->last_T, b->slot, b->traj,
+                    b->gains, b->vx, X ? b->gX : nullptr, U ? b->gU : nullptr, Vx ? b->gV : nullptr,
+                    K ? b->gK : nullptr, b->err, false, b->stream));
   if (X) TO_CK(cudaMemcpyAsync(X, b->gX, nX * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
   if (U) TO_CK(cudaMemcpyAsync(U, b->gU, nU * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
   if (Vx) TO_CK(cudaMemcpyAsync(Vx, b->gV, nX * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
@@ -946,12 +941,8 @@ int tosolve_batch_noalloc(to_problem p, int B, const double* d_x0, const int* d_
   // every other region is written before it is read
   rc = launch_solve(&w, B, d_x0, d_T, nullptr, nullptr, &o, s);
   if (rc) return rc;
-  if (d_X || d_U) {
-    const int NS = std::min(w.G, kLsWidth) + 1;
-    gather_kernel<<<gather_grid(B, (p->T_max + 1) * p->n), 256, 0, s>>>(
-        B, p->T_max, p->n, p->m, ops->rs[pi], ops->gs[pi], NS, elem, w.toff, d_T, w.slot, w.traj, w.gains, nullptr,
-        d_X, d_U, nullptr, nullptr, w.err, false);
-    TO_CK(cudaGetLastError());
-  }
+  if (d_X || d_U)
+    TO_CK(to_gather(p, pi, std::min(w.G, kLsWidth) + 1, B, w.toff, d_T, w.slot, w.traj, w.gains, nullptr, d_X, d_U, nullptr,
+                    nullptr, w.err, false, s));
   return TO_OK;
 }

@@ -97,6 +97,13 @@ int to_resolve_shape(to_problem p, const to_solver_opts* o, int B, double frac, 
 // solve allocates nothing
 int to_ensure_workspace(to_batch b, const to_solver_opts* o);
 
+// gather the results of the B instances whose first knot records are toff into
+// instance-major float64 buffers (X, U, Vx, K: each may be null): api.cu,
+// gather_kernel.  NS trajectory slots a knot; err may be null
+cudaError_t to_gather(to_problem p, int prec_idx, int NS, int B, const long long* toff, const int* T, const int* slot,
+                      const void* traj, const void* gains, const double* vx, double* X, double* U, double* Vx, double* K,
+                      const int* err, bool rows_done, cudaStream_t s);
+
 // gather the last solve's X (B x (T_max+1) x n) and U (B x T_max x m) as
 // float64 into device-visible buffers (either may be null) on stream s: the
 // padding only where the solve has written its rows there (rows_done)

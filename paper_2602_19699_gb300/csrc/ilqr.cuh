@@ -2003,12 +2003,4 @@ __global__ void prepare_kernel(int B, const int* __restrict__ T, int T_max, long
                                int* __restrict__ err, int* __restrict__ status_out, int* __restrict__ queue,
                                double* __restrict__ J_out, int* __restrict__ iters_out);
 
-__global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, int NS, int rbytes,
-                              const long long* __restrict__ toff, const int* __restrict__ T,
-                              const int* __restrict__ slot,
-                              const void* __restrict__ traj, const void* __restrict__ gains,
-                              const double* __restrict__ vx, double* __restrict__ X, double* __restrict__ U,
-                              double* __restrict__ Vx, double* __restrict__ K, const int* __restrict__ err,
-                              bool rows_done);
-
 }  // namespace to

@@ -308,11 +308,8 @@ int topoll(to_server s, uint64_t req_id, double* X, double* U, double* J, int* i
     to_problem p = L.p;
     const int pr = L.b->prec == TO_FP64 ? 0 : 1;
     const int NS = std::min(L.b->G, kLsWidth) + 1;
-    gather_kernel<<<64, 256, 0, L.copy>>>(1, p->T_max, p->n, p->m, p->ops->rs[pr], p->ops->gs[pr], NS,
-                                          pr == 0 ? 8 : 4, L.seat_toff + r.seat, L.seat_T + r.seat,
-                                          L.b->slot + r.seat, L.b->traj, L.b->gains, nullptr, X ? L.gX : nullptr,
-                                          U ? L.gU : nullptr, nullptr, nullptr, nullptr, false);
-    SV_CK(cudaGetLastError());
+    SV_CK(to_gather(p, pr, NS, 1, L.seat_toff + r.seat, L.seat_T + r.seat, L.b->slot + r.seat, L.b->traj, L.b->gains,
+                    nullptr, X ? L.gX : nullptr, U ? L.gU : nullptr, nullptr, nullptr, nullptr, false, L.copy));
     if (X) SV_CK(cudaMemcpyAsync(X, L.gX, sizeof(double) * (p->T_max + 1) * p->n, cudaMemcpyDeviceToHost, L.copy));
     if (U) SV_CK(cudaMemcpyAsync(U, L.gU, sizeof(double) * p->T_max * p->m, cudaMemcpyDeviceToHost, L.copy));
     SV_CK(cudaStreamSynchronize(L.copy));

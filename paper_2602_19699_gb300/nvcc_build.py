@@ -37,7 +37,8 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(ROOT, "include", "to.h"), __file__]
+    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))
+    return _sources() + headers + [os.path.join(ROOT, "include", "to.h"), __file__]
 
 
 def stale(checked: bool = False) -> bool:
