@@ -121,13 +121,16 @@ __global__ void prepare_kernel(int B, const int* __restrict__ T, int T_max, long
 // and slots are not valid: every output is NaN and nothing is read.  The
 // horizon and slot are clamped to their ranges before use either way.
 //
-// Bound by memory.  A block takes an instance (grid.y) and a stretch of its
-// output elements, one thread each, so that every store and, within a record,
-// every load is of consecutive addresses (a thread per knot stored 8
-// bytes every 48, and read a quadruped's 432 gains alone: reading back those
-// gains, B = 512, T = 8, took 236 us and takes 137).  rows_done: the solver has
-// written the rows up to the horizon (SolveArgs.X_out, U_out), the padding
-// remains.  I: the type of an instance's element indices (gather_shape).
+// Bound by memory.  A thread takes elements of one instance that lie a block's
+// width apart, so that every store and, within a record, every load is of
+// consecutive addresses; a block holds as many instances as their outputs leave
+// room for (gather_shape).  Kernel times for X and U, against a thread per knot
+// and against a whole block per instance: point mass B = 300 000, T = 4 56 us (60,
+// 274), B = 20 000, T = 50 46 (43, 50); planar arm B = 100 000, T = 2 18 (19, 120),
+// B = 8192, T = 400 138 (180, 140); with V_x and K, quadruped B = 512, T = 8 12 (127,
+// 11).  rows_done: the solver has written the rows up to the horizon
+// (SolveArgs.X_out, U_out), the padding remains.  I: the type of an instance's
+// element indices.
 template <class I>
 __global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, int NS, int rbytes,
                               const long long* __restrict__ toff, const int* __restrict__ T,
@@ -140,11 +143,11 @@ __global__ void gather_kernel(int B, int T_max, int n, int m, int RS, int GS, in
   const double qnan = __longlong_as_double(0x7ff8000000000000LL);
   const I e0 = (I)blockIdx.x * blockDim.x + threadIdx.x, de = (I)gridDim.x * blockDim.x;
   const I nx = ((I)T_max + 1) * n, nu = (I)T_max * m, nk = K ? nu * n : 0;
-  for (int b = blockIdx.y; b < B; b += gridDim.y) {
-    double* Xb = X ? X + (long long)b * nx : nullptr;
-    double* Ub = U ? U + (long long)b * nu : nullptr;
-    double* Vb = Vx ? Vx + (long long)b * nx : nullptr;
-    double* Kb = K ? K + (long long)b * nk : nullptr;
+  for (long long b = (long long)blockIdx.y * blockDim.y + threadIdx.y; b < B; b += (long long)gridDim.y * blockDim.y) {
+    double* Xb = X ? X + b * nx : nullptr;
+    double* Ub = U ? U + b * nu : nullptr;
+    double* Vb = Vx ? Vx + b * nx : nullptr;
+    double* Kb = K ? K + b * nk : nullptr;
     if (rejected) {
       if (X) for (I e = e0; e < nx; e += de) Xb[e] = qnan;
       if (U) for (I e = e0; e < nu; e += de) Ub[e] = qnan;
@@ -603,9 +606,9 @@ cudaError_t to_gather(to_problem p, int prec_idx, int NS, int B, const long long
   const SysOps* o = p->ops;
   const GatherShape g = gather_shape(B, gather_elems(p->T_max, p->n, p->m, K != nullptr));
   auto* kernel = g.wide ? gather_kernel<long long> : gather_kernel<int>;
-  kernel<<<dim3(g.gx, g.gy), kGatherThreads, 0, s>>>(B, p->T_max, p->n, p->m, o->rs[prec_idx], o->gs[prec_idx], NS,
-                                                     prec_idx == 0 ? 8 : 4, toff, T, slot, traj, gains, vx, X, U, Vx, K,
-                                                     err, rows_done);
+  kernel<<<dim3(g.gx, g.gy), dim3(g.bx, g.by), 0, s>>>(B, p->T_max, p->n, p->m, o->rs[prec_idx], o->gs[prec_idx], NS,
+                                                       prec_idx == 0 ? 8 : 4, toff, T, slot, traj, gains, vx, X, U, Vx,
+                                                       K, err, rows_done);
   return cudaGetLastError();
 }
 

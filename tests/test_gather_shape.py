@@ -17,7 +17,7 @@ int main(int argc, char** argv) {
   for (int i = 1; i + 4 < argc; i += 5) {
     const long long e = to::gather_elems(atoi(argv[i + 1]), atoi(argv[i + 2]), atoi(argv[i + 3]), atoi(argv[i + 4]));
     const to::GatherShape s = to::gather_shape(atoi(argv[i]), e);
-    printf("%lld %u %u %d %d\n", e, s.gx, s.gy, (int)s.wide, to::kGatherThreads);
+    printf("%lld %u %u %u %u %d %d\n", e, s.bx, s.by, s.gx, s.gy, (int)s.wide, to::kGatherThreads);
   }
 }
 """
@@ -41,11 +41,14 @@ def shapes(tmp_path_factory):
 def test_indices_fit_their_type_and_reach_every_element(shapes):
     assert len(shapes) == 3 * len(HORIZONS) * len(SYSTEMS) * 2
     kinds = set()
-    for (B, T, n, m, K), (elems, gx, gy, wide, threads) in shapes:
+    for (B, T, n, m, K), (elems, bx, by, gx, gy, wide, threads) in shapes:
         assert elems == max((T + 1) * n, T * m * n if K else 0)
-        stride = gx * threads
+        stride = gx * bx
         # a thread's last index, one stride past the output's end, and the sizes that the kernel forms
         assert elems + 2 * stride < 2 ** (63 if wide else 31), (T, n, m, K)
         assert stride >= 1 and 1 <= gy <= min(B, 65535) and gx < 2 ** 31
+        assert bx * by == threads and threads % 32 == 0
+        # a block less than twice as wide as an instance's output; no set of instances without an instance
+        assert bx < max(16, 2 * elems) and (gy - 1) * by < B
         kinds.add(wide)
     assert kinds == {0, 1}
