@@ -442,6 +442,14 @@ static int ensure_options(to_batch b, const to_solver_opts* o, bool need_uinit, 
     b->forced_cap = (size_t)b->B_max * o->max_iter;
   }
   b->bytes += extra;
+  {
+    std::lock_guard<std::mutex> lock(b->gC_mu);
+    if (b->gC && b->budget && b->bytes + b->gC_cap * sizeof(double) > b->budget) {   // a kept critic buffer makes room
+      cudaFree(b->gC);
+      b->gC = nullptr;
+      b->gC_cap = 0;
+    }
+  }
   if (b->budget && b->bytes > b->budget) return fail(TO_ERR_BUDGET, "solve: workspace exceeds the HBM budget");
   return TO_OK;
 }
@@ -784,6 +792,47 @@ int toget_trajectories(to_batch b, double* X, double* U, double* J, int* iters, 
   return TO_OK;
 }
 
+// Device memory of one toget_critic_targets call.  An allocation and a release a
+// call were most of its 190 us (B = 2048, T = 100; 78 without), so the batch
+// keeps one buffer between calls; a call that finds it taken by another
+// thread's, or too small, allocates its own.  Kept only where it fits the
+// batch's budget beside the workspace.
+struct CriticBuffer {
+  to_batch b;
+  double* d = nullptr;
+  size_t cap = 0;
+  bool keep = false;   // the call's work is done: the buffer may serve the next
+  explicit CriticBuffer(to_batch b_) : b(b_) {}
+  cudaError_t take(size_t count) {
+    {
+      std::lock_guard<std::mutex> lock(b->gC_mu);
+      if (b->gC_cap >= count) {
+        d = b->gC;
+        cap = b->gC_cap;
+        b->gC = nullptr;
+        b->gC_cap = 0;
+        return cudaSuccess;
+      }
+      if (b->gC) cudaFree(b->gC);   // too small
+      b->gC = nullptr;
+      b->gC_cap = 0;
+    }
+    const cudaError_t e = cudaMalloc(&d, count * sizeof(double));
+    if (e == cudaSuccess) cap = count;
+    return e;
+  }
+  ~CriticBuffer() {
+    if (keep && (!b->budget || b->bytes + cap * sizeof(double) <= b->budget)) {
+      std::lock_guard<std::mutex> lock(b->gC_mu);
+      if (b->gC_cap < cap) {
+        std::swap(d, b->gC);
+        std::swap(cap, b->gC_cap);
+      }
+    }
+    if (d) cudaFree(d);
+  }
+};
+
 int toget_critic_targets(to_batch b, int K, double* Vbar) {
   if (!b || !Vbar || K < 1) return fail(TO_ERR_ARG, "toget_critic_targets: null batch / output or K < 1");
   to_problem p = b->p;
@@ -792,15 +841,9 @@ int toget_critic_targets(to_batch b, int K, double* Vbar) {
   if (B == 0) return TO_OK;
   if (!b->last_T) return fail(TO_ERR_ARG, "toget_critic_targets: the batch holds no solve");
   const size_t cnt = (size_t)B * (p->T_max + 1);
-  // kept by the batch: an allocation and a release a call were most of its 190
-  // us (B = 2048, T = 100)
-  if (b->gC_cap < cnt) {
-    size_t dummy = 0;
-    b->gC_cap = 0;
-    TO_CK(grow(b->gC, 2 * cnt, dummy));
-    b->gC_cap = cnt;
-  }
-  double* d = b->gC;
+  CriticBuffer buf(b);
+  TO_CK(buf.take(2 * cnt));
+  double* d = buf.d;
   KnotCostArgs ka{};
   ka.B = B;
   ka.T_max = p->T_max;
@@ -820,6 +863,7 @@ int toget_critic_targets(to_batch b, int K, double* Vbar) {
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(Vbar, d + cnt, cnt * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  buf.keep = e == cudaSuccess;
   if (e != cudaSuccess) return fail(TO_ERR_CUDA, std::string("toget_critic_targets: ") + cudaGetErrorString(e));
   return TO_OK;
 }

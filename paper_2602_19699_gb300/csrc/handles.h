@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -61,7 +62,9 @@ struct to_batch_s {
   double* gU = nullptr;
   double* gV = nullptr;
   double* gK = nullptr;
-  // critic targets: per-knot costs and windows of the largest batch asked for so far
+  // critic targets: a buffer of gC_cap doubles that no call is using (a call takes it,
+  // and gives it or its own larger one back), or null
+  std::mutex gC_mu;
   double* gC = nullptr;
   size_t gC_cap = 0;
   unsigned long long* prof = nullptr;   // 8 per-phase cycle counters
