@@ -359,6 +359,7 @@ int torank_candidates(to_ranker r, int C, const double* x, int N, int* top_idx, 
   if (!r || !x || !top_idx || C < 1 || N < 1 || N > C) return to_fail(TO_ERR_ARG, "torank_candidates: bad arguments (1 <= N <= C)");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   if (C > r->cap_c) {
+    r->cap_c = 0;                      // (an allocation that fails leaves no capacity behind)
     for (void* q : {(void*)r->d_x, (void*)r->d_score, (void*)r->d_key})
       if (q) cudaFree(q);
     r->d_x = nullptr; r->d_score = nullptr; r->d_key = nullptr;
@@ -368,6 +369,7 @@ int torank_candidates(to_ranker r, int C, const double* x, int N, int* top_idx, 
     r->cap_c = C;
   }
   if (N > r->cap_n) {
+    r->cap_n = 0;
     if (r->d_out) cudaFree(r->d_out);
     r->d_out = nullptr;
     RK_CK(cudaMalloc(&r->d_out, sizeof(int) * N));
