@@ -422,7 +422,10 @@ static int ensure_options(to_batch b, const to_solver_opts* o, bool need_uinit, 
   if (elem > b->elem_bytes) return fail(TO_ERR_ARG, "solve: batch was created for mixed precision; FP64 needs a batch created with prec = TO_FP64");
   size_t extra = 0;
   cudaError_t e = cudaSuccess;
+  // (a capacity is cleared before its buffers are released: a growth that fails
+  // leaves none behind)
   if (b->hist_iter_cap < o->max_iter) {
+    b->hist_iter_cap = -1;
     e = grow(b->ahist, (size_t)b->B_max * std::max(o->max_iter, 1), extra);
     if (e == cudaSuccess) e = grow(b->Jhist, (size_t)b->B_max * (o->max_iter + 1), extra);
     if (e != cudaSuccess) return fail(TO_ERR_CUDA, std::string("solve: ") + cudaGetErrorString(e));
@@ -437,6 +440,7 @@ static int ensure_options(to_batch b, const to_solver_opts* o, bool need_uinit, 
     if (e != cudaSuccess) return fail(TO_ERR_CUDA, std::string("solve: ") + cudaGetErrorString(e));
   }
   if (need_forced && b->forced_cap < (size_t)b->B_max * o->max_iter) {
+    b->forced_cap = 0;
     e = grow(b->forced, (size_t)b->B_max * o->max_iter, extra);
     if (e != cudaSuccess) return fail(TO_ERR_CUDA, std::string("solve: ") + cudaGetErrorString(e));
     b->forced_cap = (size_t)b->B_max * o->max_iter;

@@ -34,3 +34,23 @@ def test_a_ranker_serves_smaller_requests_after_one_that_does_not_fit(P):
         if n == C0:
             np.testing.assert_array_equal(idx, want[0])
     r.close()
+
+
+def test_a_batch_solves_after_a_growth_that_does_not_fit(P):
+    prob = W.pointmass(seed=1)
+    B = 2000
+    b = W.make_batch(prob, B, seed=2, T=30)
+    h = P.tocreate_problem(prob.sys, prob.params, 30)
+    opts = P.to_default_opts(prec=P.TO_FP64, max_iter=3)
+    batch = P.tosolve_batch(h, b.x0, b.T, opts=opts)
+    want = P.toget_trajectories(batch), P.toget_history(batch)
+    opts.max_iter = 2 ** 30                            # histories of 25 TB
+    with pytest.raises(P.ToError) as e:
+        P.tosolve_batch(h, b.x0, b.T, opts=opts, batch=batch)
+    assert e.value.code == P.TO_ERR_CUDA
+    opts.max_iter = 3
+    got = P.toget_trajectories(P.tosolve_batch(h, b.x0, b.T, opts=opts, batch=batch)), P.toget_history(batch)
+    for k in ("X", "U", "J", "iters", "status"):
+        np.testing.assert_array_equal(got[0][k], want[0][k], err_msg=k)
+    for a, c in zip(got[1], want[1]):
+        np.testing.assert_array_equal(a, c)
