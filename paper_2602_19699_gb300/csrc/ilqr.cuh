@@ -128,7 +128,7 @@ TO_DEV long long ck(const SolveArgs& a, long long i, long long lim, int site) {
 // check sites (the report's [1])
 enum {
   CK_ORDER = 1, CK_SEAT, CK_HORIZON, CK_RECORD, CK_SLOT, CK_GAINS, CK_VX, CK_DSCR, CK_FORCED, CK_UINIT,
-  CK_HIST
+  CK_HIST, CK_ROWS
 };
 
 // per-phase clock64 accounting (tracing); one timer thread per warp / CTA
@@ -1479,15 +1479,16 @@ struct Solver {
   // these rows was no faster than the copy.
   TO_DEV static void put_rows(const Group<G>& g, const SolveArgs& a, R* traj, long long base, int T, int cur,
                               int inst) {
-    double* X = a.X_out + (long long)inst * (a.T_max + 1) * n;
-    double* U = a.U_out + (long long)inst * a.T_max * m;
+    const long long b = ck(a, inst, a.B, CK_ROWS), nx = (a.T_max + 1LL) * n, nu = (long long)a.T_max * m;
+    double* X = a.X_out + b * nx;
+    double* U = a.U_out + b * nu;
 #pragma unroll 4
     for (int e = g.lane; e < (T + 1) * n; e += G) {
       const R* r = rec(a, traj, base, e / n, cur);
-      X[e] = (double)r[e % n] + (kLo ? (double)r[n + m + e % n] : 0.0);
+      X[ck(a, e, nx, CK_ROWS)] = (double)r[e % n] + (kLo ? (double)r[n + m + e % n] : 0.0);
     }
 #pragma unroll 4
-    for (int e = g.lane; e < T * m; e += G) U[e] = (double)rec(a, traj, base, e / m, cur)[n + e % m];
+    for (int e = g.lane; e < T * m; e += G) U[ck(a, e, nu, CK_ROWS)] = (double)rec(a, traj, base, e / m, cur)[n + e % m];
   }
 
   // ------------------------------------------------------------------------
