@@ -340,120 +340,57 @@ TO_DEV void eigclip_sym3(R* Qio, R eps_in) {
     }
 }
 
-// Eigenvalue clipping of a small symmetric matrix (Sec. IV-B),
+// Eigenvalue clipping of a symmetric 3x3 matrix (Sec. IV-B),
 //   S' = max(S, eps),  Q_psd = sym(W diag(S') W^T),
-// after two exact shortcuts; 3x3 blocks then take the closed form above,
-// larger ones an in-place cyclic Jacobi eigen-decomposition (Golub & Van
-// Loan sec. 8.5).  One thread; P is row-major P x P.
-template <class R, int P>
-TO_DEV void eigclip_small(R* Q, R eps) {
-  // Two exact shortcuts before the iteration:
+// by the closed form above after two exact shortcuts.  One thread; row-major.
+template <class R>
+TO_DEV void eigclip_3x3(R* Q, R eps) {
+  constexpr int P = 3;
+  // Two exact shortcuts:
   //  * Gershgorin: if every eigenvalue is <= eps the clip is eps I;
   //  * if Q - eps I has a Cholesky factor (positive pivots) every eigenvalue
   //    is > eps and the clip is the identity map.
-  {
-    R gmax = -R(1e30);
+  R gmax = -R(1e30);
 #pragma unroll
-    for (int i = 0; i < P; ++i) {
-      R s = Q[i * P + i];
+  for (int i = 0; i < P; ++i) {
+    R s = Q[i * P + i];
 #pragma unroll
-      for (int j = 0; j < P; ++j)
-        if (j != i) s += fabs(Q[i * P + j]);
-      gmax = s > gmax ? s : gmax;
-    }
-    if (gmax <= eps) {
-#pragma unroll
-      for (int i = 0; i < P; ++i)
-#pragma unroll
-        for (int j = 0; j < P; ++j) Q[i * P + j] = (i == j) ? eps : R(0);
-      return;
-    }
-    R C[P][P];
-    bool pd = true;
-#pragma unroll
-    for (int j = 0; j < P; ++j) {
-      R s = Q[j * P + j] - eps;
-#pragma unroll
-      for (int k = 0; k < j; ++k) s -= C[j][k] * C[j][k];
-      pd = pd && (s > R(0));
-      const R r = rsqrt_(s > R(0) ? s : R(1));
-#pragma unroll
-      for (int i = j + 1; i < P; ++i) {
-        R t = Q[i * P + j];
-#pragma unroll
-        for (int k = 0; k < j; ++k) t -= C[i][k] * C[j][k];
-        C[i][j] = t * r;
-      }
-      C[j][j] = s * r;
-    }
-    if (pd) return;
+    for (int j = 0; j < P; ++j)
+      if (j != i) s += fabs(Q[i * P + j]);
+    gmax = s > gmax ? s : gmax;
   }
-  if constexpr (P == 3) {
-    eigclip_sym3(Q, eps);
+  if (gmax <= eps) {
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+#pragma unroll
+      for (int j = 0; j < P; ++j) Q[i * P + j] = (i == j) ? eps : R(0);
     return;
   }
-  R A[P][P], W[P][P];
+  R C[P][P];
+  bool pd = true;
 #pragma unroll
-  for (int i = 0; i < P; ++i)
+  for (int j = 0; j < P; ++j) {
+    R s = Q[j * P + j] - eps;
 #pragma unroll
-    for (int j = 0; j < P; ++j) { A[i][j] = Q[i * P + j]; W[i][j] = (i == j) ? R(1) : R(0); }
-  for (int sweep = 0; sweep < 12; ++sweep) {
-    R off = 0, tot = 0;
+    for (int k = 0; k < j; ++k) s -= C[j][k] * C[j][k];
+    pd = pd && (s > R(0));
+    const R r = rsqrt_(s > R(0) ? s : R(1));
 #pragma unroll
-    for (int p = 0; p < P; ++p)
+    for (int i = j + 1; i < P; ++i) {
+      R t = Q[i * P + j];
 #pragma unroll
-      for (int q = 0; q < P; ++q) {
-        tot += A[p][q] * A[p][q];
-        if (p != q) off += A[p][q] * A[p][q];
-      }
-    if (!(off > R(sizeof(R) == 4 ? 1e-14 : 1e-30) * tot)) break;   // off-diagonal below (unit roundoff)^2
-#pragma unroll
-    for (int p = 0; p < P; ++p)
-#pragma unroll
-      for (int q = p + 1; q < P; ++q) {
-        R apq = A[p][q];
-        if (apq != R(0)) {
-          R tau = (A[q][q] - A[p][p]) / (R(2) * apq);
-          R t = (tau >= R(0) ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
-          R c = rsqrt_(R(1) + t * t), s = t * c;
-#pragma unroll
-          for (int k = 0; k < P; ++k) {
-            R akp = A[k][p], akq = A[k][q];
-            A[k][p] = c * akp - s * akq;
-            A[k][q] = s * akp + c * akq;
-          }
-#pragma unroll
-          for (int k = 0; k < P; ++k) {
-            R apk = A[p][k], aqk = A[q][k];
-            A[p][k] = c * apk - s * aqk;
-            A[q][k] = s * apk + c * aqk;
-          }
-#pragma unroll
-          for (int k = 0; k < P; ++k) {
-            R wkp = W[k][p], wkq = W[k][q];
-            W[k][p] = c * wkp - s * wkq;
-            W[k][q] = s * wkp + c * wkq;
-          }
-        }
-      }
-  }
-  R S[P];
-#pragma unroll
-  for (int i = 0; i < P; ++i) S[i] = A[i][i] > eps ? A[i][i] : eps;
-#pragma unroll
-  for (int i = 0; i < P; ++i)
-#pragma unroll
-    for (int j = i; j < P; ++j) {
-      R s = 0;
-#pragma unroll
-      for (int k = 0; k < P; ++k) s += W[i][k] * S[k] * W[j][k];
-      Q[i * P + j] = s;
-      Q[j * P + i] = s;
+      for (int k = 0; k < j; ++k) t -= C[i][k] * C[j][k];
+      C[i][j] = t * r;
     }
+    C[j][j] = s * r;
+  }
+  if (pd) return;
+  eigclip_sym3(Q, eps);
 }
 
-// The same clip of a larger block by the 32 lanes of a warp: Q (P x P, shared
-// memory) in place, W scratch of the same size; on is uniform over the warp, and
+// The same clip of a larger block by the 32 lanes of a warp, by cyclic Jacobi
+// (Golub & Van Loan sec. 8.5): Q (P x P, shared memory) in place, W scratch of the
+// same size; on is uniform over the warp, and
 // the barriers are taken either way.  The scalars of a rotation are formed on
 // every lane, its rows and columns by lane k for entry k.
 template <class R, int P>

@@ -288,7 +288,7 @@ struct SysPlanar3 {
         s -= gee[0] * (ee[0] - k.P[b][0]) + gee[1] * (ee[1] - k.P[b][1]);
         Q[i * 3 + j] = s;
       }
-    eigclip_small<R, 3>(Q, eps);
+    eigclip_3x3(Q, eps);
 #pragma unroll
     for (int i = 0; i < n * n; ++i) lxx[i] = 0;
 #pragma unroll
