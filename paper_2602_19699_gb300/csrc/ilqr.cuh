@@ -598,7 +598,7 @@ struct Solver {
   // Returns true when every pivot passed the test and, with kSeeded (the
   // reciprocal pivot roots from rsqrt_newton), lies in the normal float32
   // range; otherwise the caller redoes the factor on the guarded path, which
-  // decides exactly as before.  The diagonal of L holds 1 / L_jj.
+  // decides by itself.  The diagonal of L holds 1 / L_jj.
   // ------------------------------------------------------------------------
   template <bool kSeeded, bool kShift>
   TO_DEV static bool chol_nb(const double (&Q)[m * m], double shift, double delta, double (&L)[m * m]) {
@@ -1698,7 +1698,7 @@ struct Solver {
             g.sync();
             if (bw && a.vx && a.want_vx)
               for (int i = g.lane; i < n; i += G) vx_at(a, a.vx, base + T)[i] = (double)w.v[i];
-            // (one lane used to rewrite the constant Hessians at every knot)
+            // (the constant Hessians once a pass)
             if (bw) Sys::running_consts(P, g.lane, G, (R)a.eps, w.lxx, w.lx, w.luu);
             // the knots' substep primals (bw is uniform over a group of whole warps): by the
             // group, or every lane the chains of its knots

@@ -101,10 +101,12 @@ template <int Q> constexpr size_t kRankSmem = sizeof(float) * ((size_t)kH * kStr
 
 // One tile of 8 Q candidates.  What bounds it: at Q = 16 a warp reads 6 16-byte
 // vectors for 128 multiply-adds (24 cycles of the shared-memory port against
-// 32 of the SM's FMA pipes); the earlier tile of 1 unit x 64 candidates read 16
-// for 64, and the port held it at 19 % of the FMA rate.  81 920 candidates of 6
-// inputs, whole call with its copies: 755 -> 344 us (the earlier scoring kernel
-// alone 647 us, its one-CTA selection 87 us); the same bits.
+// 32 of the SM's FMA pipes), where a tile of 1 unit x 64 candidates reads 16 for
+// 64 and the port holds it at 19 % of the FMA rate.  81 920 candidates of 6 inputs:
+// 249 us (647 with that tile), 55 % of the FP32 rate; the selection 26 us (87 by
+// one CTA), the copies 28, the whole call 345 (755).  The rest of the kernel's time
+// is 2 warps a scheduler with nothing to run while all of them evaluate tanh, wait
+// for a slice or sum the output layer.
 template <int Q>
 __global__ void __launch_bounds__(kH, 1) std_critic_kernel(int C, int n_in, const double* __restrict__ x,
                                                             const float* __restrict__ w, float* __restrict__ score,

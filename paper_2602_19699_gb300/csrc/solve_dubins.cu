@@ -27,11 +27,14 @@ typedef Dispatch<SysDubins, kDepth1, 1, 8, 16, 32> DBDispatch;
 
 // Float64 batches that leave a scheduler per instance take a whole warp: a
 // float64 warp instruction holds its scheduler's FP64 pipe for 64 cycles
-// however many lanes it serves, and 32 lanes share a knot's entries where 8
-// take columns of them.  Measured (3 iterations,
-// ms at 8 / 32 lanes, both with dense products): B = 64 3.90 / 2.97, 608 3.94 /
-// 3.14, 1216 3.96 / 4.97, 2048 4.15 / 9.77.  Beyond 4 instances an SM the pipes are shared and 8
-// lanes, four instances an instruction, win.  The sizes give the same bits.
+// however many lanes it serves, and 32 lanes share a knot's entries and the
+// running costs where 8 take columns of them.  Measured (152 SMs, 3 iterations,
+// ms at 8 / 16 / 32 lanes, 64-thread CTAs): B = 1 3.03 / 2.90 / 1.94, 64 2.92 /
+// 2.79 / 1.96, 608 2.96 / 2.83 / 2.05, 609 2.98 / 2.90 / 2.51, 912 2.98 / 3.01 /
+// 2.56, 1064 2.98 / 3.01 / 3.20, 1217 3.07 / 3.77 / 5.07, 2048 3.18 / 5.01 / 6.32.
+// The line is where every instance's warp has a scheduler of its own; 32 lanes
+// lead by less up to 6 instances an SM, which the rule leaves unused, and lose
+// beyond.  The sizes give the same bits.
 static int dubins_lanes(int prec, int B, int sms) { return prec == PREC_FP64 && B <= 4 * sms ? 32 : 8; }
 
 static SysOps make_ops() {

@@ -63,11 +63,11 @@ static cudaError_t planar3_occupancy(int prec, int G, int depth, int gpb, size_t
 static size_t planar3_knot_scratch(const double*, size_t, int) { return SysPlanar3::kDerivStride; }
 
 // Float32 batches that leave SMs idle at 8 lanes take 16: the 16 step sizes
-// then take one line-search round, and a warp's instances (2, not 4) wait for
-// each other's second round no more.  Measured (T 100..400, 3 iterations, ms
-// at 8 / 16 lanes): B = 64 4.46 / 3.30, 608 4.88 / 3.68, 2432 5.55 / 4.53,
-// 3000 6.19 / 4.56, 4000 6.70 / 6.02, 5000 6.77 / 7.14, 8192 8.76 / 11.2; 1.5
-// times the 16 instances an SM holds at once is where the batch still pays.
+// then take one line-search round, and a warp's instances (2, not 4) do not wait
+// for each other's second round.  Measured (152 SMs, T 100..400, 3 iterations, ms
+// at 8 / 16 lanes): B = 1 0.90 / 0.87, 64 4.27 / 3.14, 608 4.78 / 3.52, 2432 5.17 /
+// 4.37, 3648 5.96 / 4.61, 4000 6.05 / 5.42, 5000 6.30 / 6.92, 8192 7.36 / 10.4; the
+// line, 24 instances an SM, is 1.5 times what an SM holds at once.
 // Both sizes give the same bits in float32.  In float64 they do not (the
 // compiler fuses other multiply-adds), and the arm amplifies it.
 static int planar3_lanes(int prec, int B, int sms) { return prec == PREC_MIXED && B <= 24 * sms ? 16 : 8; }

@@ -26,11 +26,14 @@ typedef Dispatch<SysPointMass, kDepth1, 1, 8, 16, 32> PMDispatch;
 
 // Float64 batches that leave a scheduler per instance take a whole warp: a
 // float64 warp instruction holds its scheduler's FP64 pipe for 64 cycles
-// however many lanes it serves, and 32 lanes share a knot's entries where 8
-// take columns of them.  Measured (2 iterations,
-// ms at 8 / 32 lanes, both with dense products): B = 1 1.11 / 0.84, 64 1.07 /
-// 0.85, 608 1.08 / 0.89, 1216 1.10 / 1.37, 2048 1.14 / 2.66.  Beyond 4 instances an SM the pipes are shared and 8
-// lanes, four instances an instruction, win.  The sizes give the same bits.
+// however many lanes it serves, and 32 lanes share a knot's entries and the
+// running costs where 8 take columns of them.  Measured (152 SMs, 2 iterations,
+// ms at 8 / 16 / 32 lanes, 64-thread CTAs but for 8): B = 1 0.83 / 0.79 / 0.50, 64
+// 0.80 / 0.75 / 0.50, 608 0.82 / 0.77 / 0.53, 609 0.82 / 0.78 / 0.61, 912 0.82 /
+// 0.81 / 0.62, 1216 0.82 / 0.81 / 0.76, 1217 0.84 / 0.99 / 1.21, 2048 0.86 / 1.31 /
+// 1.48.  The line is where every instance's warp has a scheduler of its own; 32
+// lanes lead by less up to 8 instances an SM, which the rule leaves unused, and
+// lose beyond.  The sizes give the same bits.
 static int pointmass_lanes(int prec, int B, int sms) { return prec == PREC_FP64 && B <= 4 * sms ? 32 : 8; }
 
 static SysOps make_ops() {

@@ -50,8 +50,8 @@ static SysOps make_ops() {
   o.sys = 4;
   fill_layout<SysQuad>(o);
   o.n_groups = 2;
-  o.groups[0] = 64;   // a candidate lane's partner on the other warp factors the mass matrix
-  o.groups[1] = 32;   // one warp per instance: the partner is the candidate lane + 16
+  o.groups[0] = 64;   // 4 lanes a line-search candidate (a base that is no free body: a lane and its partner on the other warp)
+  o.groups[1] = 32;   // one warp per instance, 2 lanes a candidate (the partner: the candidate lane + 16)
   o.default_G = 64;
   o.default_gpb[0] = 1; o.default_gpb[1] = 1;
   o.accepts_actor = true;

@@ -159,8 +159,12 @@ struct SysRigid {
   static constexpr int anc(int i, int d) { return Topo::anc(i, d); }
   static constexpr int foot_body(int f) { return Topo::foot_body(f); }
 
-  // the arm's float32 solves are chaotic: code that would round otherwise than
-  // the rest of a solve was rounded before is not used there
+  // The arm's float32 solves are chaotic: after any change of rounding they can
+  // be compared with what they replace only by their distribution against the
+  // oracle.  The cheaper forms whose rounding differs (shared joint transforms,
+  // the sparse products of the mass matrix) are therefore not used there; that is
+  // a way of comparing, not a limit (13.7 ms against 16.4 for B = 2048, T = 50 to
+  // 200 with shared transforms, on the device).
   template <class R> static constexpr bool kKeepBits = KIND == RK_ARM7 && sizeof(R) == 4;
 
   // a body without mass needs no force of its own (the joints that place the
@@ -498,12 +502,12 @@ struct SysRigid {
   // as (mass, first moment h = mass * com, rotational inertia about the
   // origin); moving it to the parent frame rotates it and applies the
   // parallel-axis shift.  Bodies are ordered parents first.
-  // Eb, rb (nullable): the joint transforms of q from its bias pass.  A step
-  // evaluated each sine and cosine twice, 25 FP64 instructions a joint (float64
-  // arm, B = 304, T = 10 to 20: 8.93 -> 8.54 ms with the fused position update;
-  // quadruped, B = 512, T = 4 to 8: 6.79 -> 6.60 ms).  The
-  // float32 arm still does: with shared transforms the compiler fuses other
-  // multiply-adds, and the results are no longer the same bits.
+  // Eb, rb (nullable): the joint transforms of q from its bias pass, which save a
+  // second evaluation of each sine and cosine, 25 FP64 instructions a joint
+  // (float64 arm, B = 304, T = 10 to 20: 8.93 -> 8.54 ms with the fused position
+  // update; quadruped, B = 512, T = 4 to 8: 6.79 -> 6.60 ms).  The float32 arm
+  // evaluates them twice (kKeepBits: the compiler fuses other multiply-adds with
+  // shared ones).
   template <class R>
   TO_DEV static void mass_chol(const ParamsT<R>& P, const R* q, R* L, const R (*Eb)[9] = nullptr,
                                const R (*rb)[3] = nullptr) {
@@ -729,8 +733,9 @@ struct SysRigid {
   //   [ F^T  H ] [ qdd  ] = [ tau - bias     ]     H: 3 x 3 per leg
   // each lane eliminates its legs, the 6 x 6 Schur complement is summed and
   // solved on every lane, and the joints' accelerations follow from the axes.
-  // A substep is ~1.5 k instructions on all lanes, where a candidate lane ran
-  // ~4.4 k beside a partner's ~4 k on half of them, in a quarter of the code.
+  // A substep is ~1.5 k instructions on all lanes; by partner lanes it is ~4.4 k on
+  // a candidate's lane beside ~4 k on its partner's, half of the lanes, in four
+  // times the code.
   // Quadruped B=512 float32, T 4..8, 1 iteration, V_x: 9.7 -> 7.8 ms.
   // -------------------------------------------------------------------------
   static constexpr int kTeamSlot = 4 * N + m;      // x hi, x lo, joint torques of a candidate
@@ -1225,11 +1230,10 @@ struct SysRigid {
   // warps; on is uniform over it.  The arm's end-effector term goes through
   // forward kinematics: gradient and exact Hessian by nested dual numbers, one
   // pair of joints per lane, then the q-block is eigen-clipped by the lanes
-  // together (scratch: 2 N^2 elements).  On one lane, as it was, the 28 pairs and
-  // the Jacobi sweeps were a third of a solve: 7-DoF arm B=304 float64, T 10..20,
-  // 2 iterations, V_x 15.3 -> 9.0 ms; B=2048 float32, T 50..200, 2 iterations
-  // 27.5 -> 17.2 ms (the same bits; the kernel's code also shrank from 582 to 343
-  // KB).
+  // together (scratch: 2 N^2 elements).  On one lane the 28 pairs and the Jacobi
+  // sweeps are a third of a solve: 7-DoF arm B=304 float64, T 10..20, 2 iterations,
+  // V_x 15.3 ms there, 9.0 here; B=2048 float32, T 50..200, 2 iterations 27.5 and
+  // 17.2 ms (the same bits; 582 and 343 KB of code).
   template <class R, int G>
   TO_DEV static void terminal_group(const ParamsT<R>& P, const Group<G>& g, bool on, const R* x, R eps, R* lxx, R* lx,
                                     R* scratch) {
@@ -1317,13 +1321,15 @@ struct SysRigid {
   // elements per stored substep primal (a whole number of 16-byte chunks)
   template <class R> static constexpr int kPrimStride = (int)(((sizeof(Prim<R>) + 15) / 16 * 16) / sizeof(R));
 
-  // Line search of the quadruped's groups: candidate lane c < kStepSlots
-  // steps its rollout with lane c + G/2 as its partner (the other warp of a
-  // 64-lane group, the other half-warp of a 32-lane one), which forms and
-  // factors the mass matrix while lane c runs the bias Newton-Euler pass.
-  // Per candidate the scratch holds its substep's q and the factor.  The
-  // 7-DoF arm's candidates step alone: its 7-body mass matrix is cheap, and
-  // the partner split measured 2 % slower there in mixed mode.
+  // Line search of the quadruped's groups: every workload's base is a free body,
+  // whose candidates step by teams of lanes (cost_step_team).  For any other base,
+  // candidate lane c < kStepSlots steps its rollout with lane c + G/2 as its
+  // partner (the other warp of a 64-lane group, the other half-warp of a 32-lane
+  // one), which forms and factors the mass matrix while lane c runs the bias
+  // Newton-Euler pass; per candidate the scratch holds its substep's q and the
+  // factor (a team's slot is smaller).  The 7-DoF arm's candidates step alone: its
+  // 7-body mass matrix is cheap, and the partner split measured 2 % slower there in
+  // mixed mode.
   template <int G> static constexpr bool kGroupStep = (KIND == RK_QUAD) && G >= 32;
   static constexpr int kStepSlots = 16, kStepSlot = N + N * N;
   // the group's shared-memory scratch (the solver reserves it in its work
@@ -1798,8 +1804,9 @@ struct SysRigid {
   }
 
   // The substep primal chain of one knot on one lane, every substep's Prim
-  // stored at out + s kPrimStride (global memory): the same arithmetic as
-  // derivs' primal lane, with the mass matrix factored on this lane.
+  // stored at out + s kPrimStride (global memory), the mass matrix formed and
+  // factored on this lane: the 7-DoF arm's knots, and those of a quadruped whose
+  // base is not a free body.
   template <class R>
   TO_DEV static void primal_knot(const ParamsT<R>& P, const R* x, const R* u, R* out) {
     R q[N], qd[N], tin[N];
