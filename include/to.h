@@ -177,8 +177,9 @@ typedef struct {
                              1/4/8/16/32 planar arm, 32 arm, 64/32
                              quadruped); 0 = the totune
                              choice, else the system's default for the batch
-                             size (planar arm: 16 for float32 batches that
-                             would leave SMs idle at 8; point mass and
+                             size (planar arm: 16 for float32 batches of at
+                             most 8 instances an SM, or 16 with T_max >= 150
+                             and an iteration to do; point mass and
                              Dubins car: 32 for float64 batches of at most 4
                              instances an SM; the same bits at either).  1: one thread
                              per instance with every per-knot matrix in

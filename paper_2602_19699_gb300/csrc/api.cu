@@ -486,7 +486,7 @@ static int resolve_shape(to_problem p, const to_solver_opts* o, int B, double fr
   TO_CK(cudaGetDevice(&dev));
   TO_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (!G && !gpb && ops->lanes) {
-    G = ops->lanes(prec, B, std::max(1, (int)(sms * std::min(1.0, std::max(frac, 0.0)))));
+    G = ops->lanes(prec, B, std::max(1, (int)(sms * std::min(1.0, std::max(frac, 0.0)))), p->T_max, o->max_iter);
     if (G != ops->default_G) gpb = std::max(1, 64 / G);
   }
   if (!G) G = ops->default_G;

@@ -28,10 +28,11 @@ struct SysOps {
   int groups[6];
   int default_G, default_gpb[2];    // default launch shape (FP64, mixed)
   // lanes per instance of a solve of B instances on sms SMs that names no
-  // shape; null: default_G.  The sizes it picks from give the same bits (a
-  // result does not depend on the batch it is solved in), and each other
-  // size's CTAs have 64 threads
-  int (*lanes)(int prec, int B, int sms);
+  // shape, of at most max_iter iterations over horizons up to T_max; null:
+  // default_G.  The sizes it picks from give the same bits (a result does not
+  // depend on the batch it is solved in), and each other size's CTAs have 64
+  // threads
+  int (*lanes)(int prec, int B, int sms, int T_max, int max_iter);
   bool rows_out;                    // its groups of more than one lane write SolveArgs.X_out
   bool accepts_actor;
   // parse the flat parameter vector into the system's struct in float64 and float32

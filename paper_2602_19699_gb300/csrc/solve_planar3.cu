@@ -62,15 +62,27 @@ static cudaError_t planar3_occupancy(int prec, int G, int depth, int gpb, size_t
 // every knot's stored derivative block (both precisions)
 static size_t planar3_knot_scratch(const double*, size_t, int) { return SysPlanar3::kDerivStride; }
 
-// Float32 batches that leave SMs idle at 8 lanes take 16: the 16 step sizes
-// then take one line-search round, and a warp's instances (2, not 4) do not wait
-// for each other's second round.  Measured (152 SMs, T 100..400, 3 iterations, ms
-// at 8 / 16 lanes): B = 1 0.90 / 0.87, 64 4.27 / 3.14, 608 4.78 / 3.52, 2432 5.17 /
-// 4.37, 3648 5.96 / 4.61, 4000 6.05 / 5.42, 5000 6.30 / 6.92, 8192 7.36 / 10.4; the
-// line, 24 instances an SM, is 1.5 times what an SM holds at once.
+// Float32 batches that leave schedulers idle at 8 lanes take 16: the 16 step
+// sizes then take one line-search round, and a warp's instances (2, not 4) do not
+// wait for each other's second round.  Up to 8 instances an SM every warp of 16
+// lanes has a scheduler of its own and 16 lost nowhere; up to the 16 that an SM
+// holds at once it gains where the horizons are long and loses where they are
+// short or nothing but a rollout is asked for; beyond, the batch takes a second
+// wave that 8 lanes do not.  Measured (152 SMs, ms at 8 / 16 lanes, T the same for
+// all or drawn between two):
+//   B = 64     T 100..400 3 it. 4.32 / 3.17, T 100 3 it. 0.99 / 0.84, T 10 0.126 / 0.116
+//   B = 608    4.73 / 3.52, 1.15 / 0.93, 0.129 / 0.121
+//   B = 1216   4.79 / 3.64, 1.26 / 1.05, 0.131 / 0.128
+//   B = 1824   T 200..400 5.14 / 4.23, T 100..200 2.48 / 2.19, T 50..100 1.13 / 1.15, T 25..50 0.57 / 0.60, T 10 0.140 / 0.159,
+//              no iteration, T 400 0.238 / 0.297
+//   B = 2432   5.24 / 4.44, 2.63 / 2.28, 1.24 / 1.17, 0.60 / 0.62, 0.146 / 0.156, 0.239 / 0.297
+//   B = 3000   T 200..400 5.93 / 5.81, T 50..100 1.35 / 1.39, T 200 3.19 / 4.62, T 100 1.56 / 2.36
 // Both sizes give the same bits in float32.  In float64 they do not (the
 // compiler fuses other multiply-adds), and the arm amplifies it.
-static int planar3_lanes(int prec, int B, int sms) { return prec == PREC_MIXED && B <= 24 * sms ? 16 : 8; }
+static int planar3_lanes(int prec, int B, int sms, int T_max, int max_iter) {
+  if (prec != PREC_MIXED) return 8;
+  return B <= 8 * sms || (B <= 16 * sms && T_max >= 150 && max_iter > 0) ? 16 : 8;
+}
 
 static SysOps make_ops() {
   SysOps o{};

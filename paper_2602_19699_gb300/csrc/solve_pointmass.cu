@@ -34,7 +34,7 @@ typedef Dispatch<SysPointMass, kDepth1, 1, 8, 16, 32> PMDispatch;
 // 1.48.  The line is where every instance's warp has a scheduler of its own; 32
 // lanes lead by less up to 8 instances an SM, which the rule leaves unused, and
 // lose beyond.  The sizes give the same bits.
-static int pointmass_lanes(int prec, int B, int sms) { return prec == PREC_FP64 && B <= 4 * sms ? 32 : 8; }
+static int pointmass_lanes(int prec, int B, int sms, int, int) { return prec == PREC_FP64 && B <= 4 * sms ? 32 : 8; }
 
 static SysOps make_ops() {
   SysOps o{};
