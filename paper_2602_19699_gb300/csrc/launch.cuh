@@ -64,8 +64,17 @@ int multi_group_lanes(int slot);       // lanes per instance of the slot's solve
 
 constexpr int kMaxCtaThreads = 256;
 
+// CTAs of the largest size that the registers must leave room for on an SM.  The
+// point mass's and the car's float32 kernels at 16 and 32 lanes are bound by the
+// warps in flight once the batch fills the GPU; without the cap they take 148 to
+// 181 registers (120 to 124 with it, no spills), and lose to what that leaves
+// resident: point mass, B = 20 000, T = 50, 3 iterations, 32 lanes 7.15 ms, capped 4.96;
+// B = 4000, 16 lanes 0.69 and 0.46.
+template <class Sys, class R, int G>
+constexpr int min_ctas() { return Sys::kGainDerivs && sizeof(R) == 4 && G >= 16 ? 2 : 1; }
+
 template <class Sys, class R, int G, int D>
-__global__ void __launch_bounds__(kMaxCtaThreads, 1) ilqr_kernel(SolveArgs a) {
+__global__ void __launch_bounds__(kMaxCtaThreads, min_ctas<Sys, R, G>()) ilqr_kernel(SolveArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Solver<Sys, R, G, D>::run(a, smem_raw);
 }
