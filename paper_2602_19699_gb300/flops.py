@@ -1,7 +1,10 @@
 """Algorithmic floating-point work of one iLQR solve, for the roofline.
 
 Counts are FP adds, multiplies and FMAs (an FMA counts 2; sqrt, rsqrt, sin,
-cos and exp count 1 each) of the minimal formulation of each step, per knot:
+cos and exp count 1 each) of a plain formulation of each step, per knot.  They
+are a fixed reference: kernels that skip zeros (the point mass's and the car's
+products) or share a step among lanes (the quadruped's line search) execute
+less than is counted here:
 
 * backward Riccati step (Sec. II; Sec. IV-B's clip excluded):
     V A (2n^3) + V B (2n^2 m) + A^T (V A) upper triangle (n^2 (n+1))
