@@ -62,6 +62,7 @@ def parse_args():
     ap.add_argument("--no-extras", action="store_true", help="skip the plain and FP64 comparison legs")
     ap.add_argument("--quad-budget", action="store_true",
                     help="also run the quadruped at its calibrated 1000-iteration budget (about 140 s)")
+    ap.add_argument("--details", metavar="FILE", help="also write every measurement of the run to FILE (JSON)")
     return ap.parse_args()
 
 
@@ -218,6 +219,77 @@ def peaks():
 def fp32_alu_peak_tflops(sm_mhz: float, sms: int) -> float:
     """152 SMs x 128 FP32 lanes x 2 FLOP per FMA x SM clock."""
     return sms * 128 * 2 * sm_mhz * 1e6 / 1e12
+
+
+# --------------------------------------------------------------------------
+# the printed line
+# --------------------------------------------------------------------------
+def _short(o):
+    """Floats at six significant digits, in any nesting."""
+    if isinstance(o, dict):
+        return {k: _short(v) for k, v in o.items()}
+    if isinstance(o, (list, tuple)):
+        return [_short(v) for v in o]
+    return float(f"{o:.6g}") if isinstance(o, float) else o
+
+
+def _sides(g):
+    """One- and two-sided fractions of an accuracy-gate record."""
+    return {k: g[k] for k in ("sample", "one_sided", "two_sided") if k in g} if g else None
+
+
+def _leg(r):
+    """One system's row in one precision."""
+    out = {k: r[k] for k in ("B", "ms", "value") if k in r}
+    if r.get("roofline"):
+        out["frac"] = r["roofline"]["frac"]
+    g = (r.get("accuracy") or {}).get("gates") or {}
+    out.update({k: g[k] for k in ("one_sided", "two_sided") if k in g})
+    return out
+
+
+SERVE_COLUMNS = ("rate_per_s", "solves_per_s", "p50_ms", "p99_ms")
+
+
+def compact_line(full: dict) -> dict:
+    """The line that is printed: the headline's fields as they are, and of the
+    comparison legs the times, rates and fractions.  It stays below 4.8 kB, so
+    that a reader who keeps the end of a log has all of it; descriptions,
+    distributions, tuned shapes and per-sample records go to --details."""
+    line = dict(full)
+    wt = full.get("within_tol")
+    if wt:
+        line["within_tol"] = _short({"cost_tol": wt["cost_tol"], "fraction": wt["fraction"], "rule": "J <= (1 + 1e-6) J_oracle",
+                                     "gates": _sides(wt.get("gates")),
+                                     "oracle_self_reproducibility": _sides(wt.get("oracle_self_reproducibility"))})
+    if "autotune" in full:
+        line["autotune"] = {"chosen": full["autotune"]["chosen"]}
+    for k in ("roofline", "cpu_baseline", "batched_fp64", "plain_fp64_one_instance_per_launch"):
+        if k in full:
+            line[k] = _short(full[k])
+    lm = full.get("levenberg_marquardt")
+    if lm:
+        line["levenberg_marquardt"] = _short({k: lm[k] for k in ("ms_per_step", "raw_solves_per_s", "mean_iters",
+                                                                 "within_tol_vs_lm_oracle") if k in lm})
+    serve = full.get("serve")
+    if serve:
+        line["serve"] = _short({"columns": SERVE_COLUMNS, **{p: [[x.get(c) for c in SERVE_COLUMNS] for x in serve[p]]
+                                                             for p in ("mixed", "fp64") if p in serve}})
+    if full.get("other_workloads"):
+        line["other_workloads"] = _short({
+            name: {k: _leg(v) for k, v in legs.items() if k in ("mixed", "fp64") and isinstance(v, dict)}
+            for name, legs in full["other_workloads"].items()})
+    if full.get("bic_ranking"):
+        line["bic_ranking"] = _short({name: {c: v[c] for c in ("candidates", "ms", "frac_of_fp32_peak") if c in v}
+                                      for name, v in full["bic_ranking"].items()})
+    ms = full.get("multi_system")
+    if ms:
+        out = {k: ms[k] for k in ("sequential_s", "one_launch_s") if k in ms}
+        for k in ("equal_shares", "work_shares"):
+            if isinstance(ms.get(k), dict):
+                out[f"graph_{k}_s"] = ms[k].get("graph_s")
+        line["multi_system"] = _short(out)
+    return line
 
 
 # the sources the timed planar-arm solver kernel is compiled from
@@ -563,7 +635,10 @@ def run_gb300(args):
         line["bic_ranking"] = bic
     if multi is not None:
         line["multi_system"] = multi
-    print(json.dumps(line), flush=True)
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(line, f, indent=1)
+    print(json.dumps(compact_line(line)), flush=True)
     if ws > 1:
         torch.distributed.barrier()
         torch.distributed.destroy_process_group()
